@@ -27,10 +27,23 @@
 namespace cwell {
 
 // ------------------------------------------------------------------ GEMM
-// C[M x N] = alpha * op(A)[M x K] * op(B)[K x N] + beta * C, A and B BF16
-// row-major (op = transpose when TA / TB), C FP32 row-major.  64 x 64 tiles,
-// K step 32, four warps of 32 x 32, mma.sync m16n8k16 (BF16 in, FP32 acc).
-constexpr int GBM = 64, GBN = 64, GBK = 32, GPAD = 8;
+// C[M x N] = op(A)[M x K] * op(B)[K x N], A and B BF16 row-major (op =
+// transpose when TA / TB), C FP32 row-major.  64 x 64 tiles, K step 32, four
+// warps of 32 x 32, mma.sync m16n8k16 (BF16 in, FP32 acc).
+//
+// The products here have a few MFLOP, so what bounds them is the latency of
+// one block's walk along K.  Operand tiles are staged four deep with 16-byte
+// cp.async in the layout of their source ([row][k] or [k][row]; ldmatrix,
+// transposing where K is not the contiguous index, forms the fragments), so
+// three K steps of loads are in flight behind the MMAs (64 x 512 x 256 in 6.7
+// us, 32 x 512 x 4096 in 54 us; 43 and 573 us with 2-byte loads staged one K
+// step at a time).  Every element is one
+// chain of MMAs over ascending K, as in gemm_wgrad below: the training
+// amplifies a changed order of the sum (Adam divides by the gradients' own
+// size), so no product is cut along K.
+constexpr int GBM = 64, GBN = 64, GBK = 32, GST = 4;
+constexpr int GLD_K = GBK + 8, GLD_R = 64 + 8;  // row pitch of a [row][k] / [k][row] tile: ldmatrix rows in distinct banks
+constexpr int GTILE = GBM * GLD_K;              // elements per staged tile (the larger of the two layouts)
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
   asm volatile(
@@ -40,55 +53,101 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  if (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+// Stage a 64 (rows r0 .. of R) x 32 (k0 .. of kend) operand tile: KC = K is
+// the contiguous index of the source (element (r, k) at src[r ld + k], tile
+// [row][k]), otherwise element (r, k) at src[k ld + r], tile [k][row].  Eight
+// contiguous elements at a time, zero outside; vec: rows of the source are
+// 16-byte aligned (ld a multiple of 8, base aligned).
+template <bool KC>
+__device__ __forceinline__ void stage_tile(__nv_bfloat16 *tile, const __nv_bfloat16 *src, int ld, int r0, int R, int k0,
+                                           int kend, bool vec) {
+#pragma unroll
+  for (int q = threadIdx.x; q < 256; q += 128) {
+    const int r = KC ? q >> 2 : (q & 7) * 8, k = KC ? (q & 3) * 8 : q >> 3;
+    const int gr = r0 + r, gk = k0 + k;
+    const int left = KC ? kend - gk : R - gr;  // elements of the source row from here on
+    const bool in = KC ? gr < R : gk < kend;
+    const int n = in ? max(0, min(8, left)) : 0;
+    const __nv_bfloat16 *g = n > 0 ? src + (KC ? (long long)gr * ld + gk : (long long)gk * ld + gr) : src;
+    __nv_bfloat16 *d = tile + (KC ? r * GLD_K + k : k * GLD_R + r);
+    if (vec) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(d)), "l"(g),
+                   "r"(2 * n)
+                   : "memory");
+    } else {
+      uint32_t w[4];
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        const uint32_t lo = 2 * e < n ? __bfloat16_as_ushort(g[2 * e]) : 0u;
+        const uint32_t hi = 2 * e + 1 < n ? __bfloat16_as_ushort(g[2 * e + 1]) : 0u;
+        w[e] = lo | (hi << 16);
+      }
+      *reinterpret_cast<uint4 *>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+}
+
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(128) gemm_bf16(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda,
                                                  const __nv_bfloat16 *__restrict__ B, int ldb, float *__restrict__ C,
-                                                 int ldc, float alpha, float beta) {
-  __shared__ __align__(16) __nv_bfloat16 As[GBM][GBK + GPAD];
-  __shared__ __align__(16) __nv_bfloat16 Bs[GBN][GBK + GPAD];
+                                                 int ldc) {
+  __shared__ __align__(16) __nv_bfloat16 As[GST][GTILE], Bs[GST][GTILE];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
   const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-  const int g = lane >> 2, t = lane & 3;
+  const int nk = (K + GBK - 1) / GBK;
+  const bool va = (lda % 8) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  const bool vb = (ldb % 8) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+  auto stage = [&](int c) {
+    if (c < nk) {
+      stage_tile<!TA>(As[c % GST], A, lda, m0, M, c * GBK, K, va);
+      stage_tile<TB>(Bs[c % GST], B, ldb, n0, N, c * GBK, K, vb);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int c = 0; c < GST - 1; c++) stage(c);
   float acc[2][4][4] = {};
-  const __nv_bfloat16 zero = __float2bfloat16(0.f);
-  for (int k0 = 0; k0 < K; k0 += GBK) {
-    // stage op(A)[m0.., k0..] as As[m][k] and op(B)[k0.., n0..] as Bs[n][k]
-    for (int q = tid; q < GBM * GBK; q += 128) {
-      const int mm = TA ? q % GBM : q / GBK, kk = TA ? q / GBM : q % GBK;
-      const int m = m0 + mm, k = k0 + kk;
-      As[mm][kk] = (m < M && k < K) ? (TA ? A[(long long)k * lda + m] : A[(long long)m * lda + k]) : zero;
-    }
-    for (int q = tid; q < GBN * GBK; q += 128) {
-      const int nn = TB ? q / GBK : q % GBN, kk = TB ? q % GBK : q / GBN;
-      const int n = n0 + nn, k = k0 + kk;
-      Bs[nn][kk] = (n < N && k < K) ? (TB ? B[(long long)n * ldb + k] : B[(long long)k * ldb + n]) : zero;
-    }
-    __syncthreads();
+  for (int c = 0; c < nk; c++) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(GST - 2) : "memory");
+    __syncthreads();  // tile c has landed for every thread, and all are done with the slot refilled next
+    stage(c + GST - 1);
+    const __nv_bfloat16 *a_s = As[c % GST], *b_s = Bs[c % GST];
 #pragma unroll
     for (int ks = 0; ks < GBK; ks += 16) {
-      uint32_t af[2][4], bfr[4][2];
+      uint32_t af[2][4], bp[2][4];
 #pragma unroll
       for (int i = 0; i < 2; i++) {
-        const int r = wm + 16 * i + g;
-        af[i][0] = *reinterpret_cast<const uint32_t *>(&As[r][ks + 2 * t]);
-        af[i][1] = *reinterpret_cast<const uint32_t *>(&As[r + 8][ks + 2 * t]);
-        af[i][2] = *reinterpret_cast<const uint32_t *>(&As[r][ks + 2 * t + 8]);
-        af[i][3] = *reinterpret_cast<const uint32_t *>(&As[r + 8][ks + 2 * t + 8]);
+        const int r = wm + 16 * i, lo = lane & 7, mid = ((lane >> 3) & 1) * 8, hi = (lane >> 4) * 8;
+        ldsm4<TA>(af[i], TA ? a_s + (ks + lo + hi) * GLD_R + r + mid : a_s + (r + lo + mid) * GLD_K + ks + hi);
       }
 #pragma unroll
-      for (int j = 0; j < 4; j++) {
-        const int c = wn + 8 * j + g;
-        bfr[j][0] = *reinterpret_cast<const uint32_t *>(&Bs[c][ks + 2 * t]);
-        bfr[j][1] = *reinterpret_cast<const uint32_t *>(&Bs[c][ks + 2 * t + 8]);
+      for (int j = 0; j < 2; j++) {  // 16 columns: two 8-column fragments
+        const int r = wn + 16 * j, lo = lane & 7, mid = ((lane >> 3) & 1) * 8, hi = (lane >> 4) * 8;
+        ldsm4<!TB>(bp[j], TB ? b_s + (r + lo + hi) * GLD_K + ks + mid : b_s + (ks + lo + mid) * GLD_R + r + hi);
       }
 #pragma unroll
       for (int i = 0; i < 2; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) mma_bf16(acc[i][j], af[i], bfr[j]);
+        for (int j = 0; j < 4; j++) {
+          const uint32_t bf[2] = {bp[j >> 1][(j & 1) * 2], bp[j >> 1][(j & 1) * 2 + 1]};
+          mma_bf16(acc[i][j], af[i], bf);
+        }
     }
-    __syncthreads();
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  const int g = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int i = 0; i < 2; i++)
 #pragma unroll
@@ -97,22 +156,18 @@ __global__ void __launch_bounds__(128) gemm_bf16(int M, int N, int K, const __nv
       for (int e = 0; e < 4; e++) {
         const int m = m0 + wm + 16 * i + g + (e >= 2 ? 8 : 0);
         const int n = n0 + wn + 8 * j + 2 * t + (e & 1);
-        if (m < M && n < N) {
-          float *cp = C + (long long)m * ldc + n;
-          *cp = alpha * acc[i][j][e] + (beta != 0.f ? beta * *cp : 0.f);
-        }
+        if (m < M && n < N) C[(long long)m * ldc + n] = acc[i][j][e];
       }
 }
 
 static cudaError_t gemm_mma(bool ta, bool tb, int M, int N, int K, const __nv_bfloat16 *A, int lda,
-                            const __nv_bfloat16 *B, int ldb, float *C, int ldc, float alpha, float beta,
-                            cudaStream_t s) {
+                            const __nv_bfloat16 *B, int ldb, float *C, int ldc, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   dim3 grd((N + GBN - 1) / GBN, (M + GBM - 1) / GBM);
-  if (!ta && !tb) gemm_bf16<false, false><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta);
-  else if (!ta && tb) gemm_bf16<false, true><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta);
-  else if (ta && !tb) gemm_bf16<true, false><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta);
-  else gemm_bf16<true, true><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta);
+  if (!ta && !tb) gemm_bf16<false, false><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc);
+  else if (!ta && tb) gemm_bf16<false, true><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc);
+  else if (ta && !tb) gemm_bf16<true, false><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc);
+  else gemm_bf16<true, true><<<grd, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc);
   return cudaGetLastError();
 }
 
@@ -121,16 +176,100 @@ static cudaError_t gemm_mma(bool ta, bool tb, int M, int N, int K, const __nv_bf
 // ones (weight gradients: rows = channels) on the mma.sync kernel above.
 // path: 0 = by shape, 1 = mma.sync, 2 = tcgen05.
 static cudaError_t gemm_path(int path, bool ta, bool tb, int M, int N, int K, const __nv_bfloat16 *A, int lda,
-                             const __nv_bfloat16 *B, int ldb, float *C, int ldc, float alpha, float beta,
-                             cudaStream_t s) {
+                             const __nv_bfloat16 *B, int ldb, float *C, int ldc, cudaStream_t s) {
   const bool tc = path == 2 || (path == 0 && M >= 128);
-  return tc ? gemm_tcgen05(ta, tb, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, s)
-            : gemm_mma(ta, tb, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, s);
+  return tc ? gemm_tcgen05(ta, tb, M, N, K, A, lda, B, ldb, C, ldc, 1.f, 0.f, s)
+            : gemm_mma(ta, tb, M, N, K, A, lda, B, ldb, C, ldc, s);
 }
 
 static cudaError_t gemm(bool ta, bool tb, int M, int N, int K, const __nv_bfloat16 *A, int lda,
-                        const __nv_bfloat16 *B, int ldb, float *C, int ldc, float alpha, float beta, cudaStream_t s) {
-  return gemm_path(0, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, s);
+                        const __nv_bfloat16 *B, int ldb, float *C, int ldc, cudaStream_t s) {
+  return gemm_path(0, ta, tb, M, N, K, A, lda, B, ldb, C, ldc, s);
+}
+
+// Weight gradients C[M x N] = A^T B, A [K][M], B [K][N] row-major with K =
+// batch x length (up to 131072) and M, N the channels (16 .. 64, 8 .. 256):
+// one output tile, a very long K.  The sum keeps its order (one chain of MMAs
+// per element, ascending K), so what bounds the kernel is the chain, K / 16
+// dependent mma.sync.  Therefore one m16n8 tile per warp (16 x 32 per block,
+// as many chains side by side as the product has), nothing in the chain but
+// the mma (each 32-row round's fragments are loaded during the round before),
+// and three stages of 256 K rows of cp.async ahead of it.  16 x 8 over K =
+// 65536: 0.18 ms, 43 ns per MMA, against 8.3 ms on the 64 x 64 tile kernel
+// staged with 2-byte loads.
+constexpr int WG_M = 16, WG_N = 32, WG_K = 256, WG_ST = 4;
+constexpr int WG_LDA = WG_M + 8, WG_LDB = WG_N + 8;  // row pitches 48 and 80 bytes: ldmatrix rows in distinct banks
+constexpr int WG_STAGE = WG_K * (WG_LDA + WG_LDB);   // elements
+constexpr int WG_SMEM = WG_ST * WG_STAGE * 2;
+
+__global__ void __launch_bounds__(128) gemm_wgrad(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda,
+                                                  const __nv_bfloat16 *__restrict__ B, int ldb, float *__restrict__ C,
+                                                  int ldc) {
+  extern __shared__ __align__(16) __nv_bfloat16 sm[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.y * WG_M, n0 = blockIdx.x * WG_N;
+  const int nk = (K + WG_K - 1) / WG_K;
+  auto copy = [&](__nv_bfloat16 *d, const __nv_bfloat16 *base, int ld, int k, int c, int cols) {
+    const int n = k < K ? max(0, min(8, cols - c)) : 0;  // elements in range, the rest is zero
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(d)),
+                 "l"(n > 0 ? base + (long long)k * ld + c : base), "r"(2 * n)
+                 : "memory");
+  };
+  auto stage = [&](int c) {
+    if (c < nk) {
+      __nv_bfloat16 *a = sm + (c % WG_ST) * WG_STAGE, *b = a + WG_K * WG_LDA;
+#pragma unroll
+      for (int q = tid; q < WG_K * 2; q += 128) copy(a + (q >> 1) * WG_LDA + (q & 1) * 8, A, lda, c * WG_K + (q >> 1), m0 + (q & 1) * 8, M);
+#pragma unroll
+      for (int q = tid; q < WG_K * 4; q += 128) copy(b + (q >> 2) * WG_LDB + (q & 3) * 8, B, ldb, c * WG_K + (q >> 2), n0 + (q & 3) * 8, N);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int c = 0; c < WG_ST - 1; c++) stage(c);
+  float acc[4] = {};
+  for (int c = 0; c < nk; c++) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(WG_ST - 2) : "memory");
+    __syncthreads();
+    stage(c + WG_ST - 1);
+    const __nv_bfloat16 *a = sm + (c % WG_ST) * WG_STAGE, *b = a + WG_K * WG_LDA + warp * 8;
+    uint32_t af[2][2][4], bf[2][4];
+    auto frags = [&](int r) {  // fragments of the 32 K rows of round r
+      ldsm4<true>(bf[r & 1], b + (32 * r + lane) * WG_LDB);
+#pragma unroll
+      for (int h = 0; h < 2; h++)
+        ldsm4<true>(af[r & 1][h], a + (32 * r + 16 * h + (lane & 7) + (lane >> 4) * 8) * WG_LDA + ((lane >> 3) & 1) * 8);
+    };
+    frags(0);
+#pragma unroll
+    for (int r = 0; r < WG_K / 32; r++) {
+      if (r + 1 < WG_K / 32) frags(r + 1);
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        const uint32_t bh[2] = {bf[r & 1][2 * h], bf[r & 1][2 * h + 1]};
+        mma_bf16(acc, af[r & 1][h], bh);
+      }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    const int m = m0 + (lane >> 2) + (e >= 2 ? 8 : 0), n = n0 + warp * 8 + 2 * (lane & 3) + (e & 1);
+    if (m < M && n < N) C[(long long)m * ldc + n] = acc[e];
+  }
+}
+
+// C = A^T B of the backward pass: gemm_wgrad where the rows are channels (M <
+// 128, as gemm_path's narrow products), 16-byte aligned, and K is long enough
+// for the stages to fill; otherwise by shape.
+static cudaError_t gemm_grad(int M, int N, int K, const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb,
+                             float *C, cudaStream_t s) {
+  const bool vec = lda % 8 == 0 && ldb % 8 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0;
+  if (M >= 128 || K < 2 * WG_K || !vec) return gemm(true, false, M, N, K, A, lda, B, ldb, C, N, s);
+  cudaError_t e = cudaFuncSetAttribute(gemm_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM);
+  if (e != cudaSuccess) return e;
+  gemm_wgrad<<<dim3((N + WG_N - 1) / WG_N, (M + WG_M - 1) / WG_M), 128, WG_SMEM, s>>>(M, N, K, A, lda, B, ldb, C, N);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ elementwise
@@ -190,44 +329,85 @@ __global__ void k_gelu_bwd(const float *da, const float *pre, long long n, float
   GRID_STRIDE(q, n) {
     const float v = da[q] * gelu_df(pre[q]);
     dz[q] = v;
-    if (dz16) dz16[q] = __float2bfloat16(v);
+    dz16[q] = __float2bfloat16(v);
   }
 }
 
-// im2col of the transposed convolution's gradient: dZ[b][s][co*4+q] = dy[b][2s-1+q][co]
-__global__ void k_im2col(const float *dy, int B, int Lin, int Cout, __nv_bfloat16 *dZ) {
+// Backward of one transposed convolution's activation: v[b][t][co] = da *
+// gelu'(pre) and its im2col dZ[b][s][co*4+q] = v[b][2s-1+q][co] (BF16, zero
+// outside), v itself in FP32 for the bias gradient.  One thread per (b, s, co)
+// reads the four outputs its taps land on (each of them twice over the
+// launch, the second time from L1) and writes its four dZ values as one
+// 8-byte word, which saves the write and two reads of v a separate im2col made.
+__global__ void k_conv_bwd(const float *__restrict__ da, const float *__restrict__ pre, int B, int Lin, int Cout,
+                           float *__restrict__ dz, __nv_bfloat16 *__restrict__ dZ) {
   const int Lout = 2 * Lin;
-  GRID_STRIDE(q, (long long)B * Lin * Cout * 4) {
-    const int cq = (int)(q % (Cout * 4));
-    const long long bs = q / (Cout * 4);
+  GRID_STRIDE(q, (long long)B * Lin * Cout) {
+    const int co = (int)(q % Cout);
+    const long long bs = q / Cout;
     const int s = (int)(bs % Lin), b = (int)(bs / Lin);
-    const int co = cq >> 2, tap = cq & 3, t = 2 * s - 1 + tap;
-    dZ[q] = __float2bfloat16((t >= 0 && t < Lout) ? dy[((long long)b * Lout + t) * Cout + co] : 0.f);
+    __nv_bfloat16 h[4];
+#pragma unroll
+    for (int tap = 0; tap < 4; tap++) {
+      const int t = 2 * s - 1 + tap;
+      const long long o = ((long long)b * Lout + t) * Cout + co;
+      float v = 0.f;
+      if (t >= 0 && t < Lout) {
+        v = da[o] * gelu_df(pre[o]);
+        if (tap == 1 || tap == 2) dz[o] = v;
+      }
+      h[tap] = __float2bfloat16(v);
+    }
+    uint2 u;
+    u.x = (uint32_t)__bfloat16_as_ushort(h[0]) | ((uint32_t)__bfloat16_as_ushort(h[1]) << 16);
+    u.y = (uint32_t)__bfloat16_as_ushort(h[2]) | ((uint32_t)__bfloat16_as_ushort(h[3]) << 16);
+    *reinterpret_cast<uint2 *>(dZ + 4 * q) = u;
   }
 }
 
-// column sums of a [rows][N] FP32 matrix into out[N] (fixed order: per-column
-// partial sums over row blocks, then a sum of the partials)
-__global__ void k_colsum_partial(const float *X, long long rows, int N, int chunk, float *part) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  const long long r0 = (long long)blockIdx.y * chunk;
-  if (n >= N) return;
+// Column sums of a [rows][N] FP32 matrix into out[N], in a fixed order: per
+// column, sums over consecutive chunks of rows, then the sum of those.  Block
+// = 128 threads over (column, chunk) pairs, column fastest, so that narrow
+// matrices (8 .. 64 columns) still fill the warps; both loops keep 16 loads
+// in flight ahead of their serial additions.
+__global__ void __launch_bounds__(128) k_colsum_partial(const float *X, long long rows, int N, int chunk, int parts,
+                                                        float *part) {
+  const long long q = blockIdx.x * 128LL + threadIdx.x;
+  if (q >= (long long)N * parts) return;
+  const int n = (int)(q % N);
+  const long long r0 = q / N * chunk, r1 = min(rows, r0 + chunk);
   float acc = 0.f;
-  for (long long r = r0; r < r0 + chunk && r < rows; r++) acc += X[r * N + n];
-  part[(long long)blockIdx.y * N + n] = acc;
+  long long r = r0;
+  for (; r + 16 <= r1; r += 16) {
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) v[e] = X[(r + e) * N + n];
+#pragma unroll
+    for (int e = 0; e < 16; e++) acc += v[e];
+  }
+  for (; r < r1; r++) acc += X[r * N + n];
+  part[q] = acc;
 }
-__global__ void k_colsum_final(const float *part, int parts, int N, float *out) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32) k_colsum_final(const float *part, int parts, int N, float *out) {
+  const int n = blockIdx.x * 32 + threadIdx.x;
   if (n >= N) return;
   float acc = 0.f;
-  for (int p = 0; p < parts; p++) acc += part[(long long)p * N + n];
+  int p = 0;
+  for (; p + 16 <= parts; p += 16) {
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) v[e] = part[(long long)(p + e) * N + n];
+#pragma unroll
+    for (int e = 0; e < 16; e++) acc += v[e];
+  }
+  for (; p < parts; p++) acc += part[(long long)p * N + n];
   out[n] = acc;
 }
 
 // MSE of channels-last predictions y[b][t][c] against targets T[b][c][t]:
 // loss partials per block, gradient dy = 2 (y - T) / count
 __global__ void k_mse(const float *y, const float *T, int B, int L, int Cc, float inv_count, float inv_ys, float *dy,
-                      float *loss_part) {
+                      __nv_bfloat16 *dy16, float *loss_part) {
   __shared__ float red[256];
   float acc = 0.f;
   GRID_STRIDE(q, (long long)B * L * Cc) {
@@ -235,7 +415,9 @@ __global__ void k_mse(const float *y, const float *T, int B, int L, int Cc, floa
     const long long bt = q / Cc;
     const int t = (int)(bt % L), b = (int)(bt / L);
     const float e = y[q] - T[((long long)b * Cc + c) * L + t] * inv_ys;
-    if (dy) dy[q] = 2.f * e * inv_count;
+    const float d = 2.f * e * inv_count;
+    dy[q] = d;
+    dy16[q] = __float2bfloat16(d);
     acc += e * e;
   }
   red[threadIdx.x] = acc;
@@ -314,6 +496,9 @@ static int egrid(long long n) { return (int)std::min<long long>((n + 255) / 256,
 // ======================================================================= host
 using namespace cwell;
 
+constexpr int COLSUM_PARTS = 4096;  // at most this many row chunks per column sum
+constexpr int LOSS_PARTS = 1024;    // blocks of the loss kernel
+
 struct sur_s {
   sur_cfg_t cfg{};
   cudaStream_t stream = nullptr;
@@ -332,9 +517,20 @@ struct sur_s {
   std::vector<float *> pre;             // per layer pre-activations (FP32)
   std::vector<__nv_bfloat16 *> act;     // per layer activations (BF16), act[0] = normalised input
   float *z = nullptr, *y = nullptr, *dy = nullptr, *da = nullptr, *dz = nullptr, *part = nullptr, *lossp = nullptr;
-  __nv_bfloat16 *dz16 = nullptr, *dy16 = nullptr;
+  __nv_bfloat16 *dy16 = nullptr;
+  // backward: per layer the gradient of its pre-activation (FP32) and the BF16 operand of its weight gradient
+  std::vector<float *> gz;
+  std::vector<__nv_bfloat16 *> gz16;
+  // The weight and bias gradients hang off the chain of data gradients and
+  // are themselves long serial sums, so they run beside it: side[0] the bias
+  // sums, side[1] the last layer's weight gradient (the longest), side[2] the
+  // others.  ready[q] marks operand q on the handle's stream, done[k] the end
+  // of side[k]; the handle's stream waits for all of them before a backward
+  // pass returns.
+  static constexpr int SIDES = 3, MAX_READY = 12;
+  cudaStream_t side[SIDES] = {};
+  cudaEvent_t done[SIDES] = {}, ready[MAX_READY] = {};
   float *xb = nullptr, *tb = nullptr;
-  int *idx = nullptr;
   std::vector<void *> allocs;
   std::vector<float> gate_x, gate_err;  // normalised validation inputs and their errors
   std::string err;
@@ -403,6 +599,15 @@ static void layout(sur_t *s) {
   s->nparam = o;
 }
 
+static void release_side(sur_t *s) {
+  for (cudaStream_t x : s->side)
+    if (x) cudaStreamDestroy(x);
+  for (cudaEvent_t x : s->done)
+    if (x) cudaEventDestroy(x);
+  for (cudaEvent_t x : s->ready)
+    if (x) cudaEventDestroy(x);
+}
+
 extern "C" int sur_create(const sur_cfg_t *cfg, const sim_opts_t *opts, sur_t **out) {
   if (!out) return sfail(nullptr, SIM_EINVAL, "out is null");
   *out = nullptr;
@@ -417,6 +622,7 @@ extern "C" int sur_create(const sur_cfg_t *cfg, const sim_opts_t *opts, sur_t **
   s->device = opts ? opts->device : 0;
   auto bail = [&](int rc) {
     g_sur_err = s->err;
+    release_side(s);
     for (void *p : s->allocs) cudaFree(p);
     if (s->own_stream) cudaStreamDestroy(s->stream);
     delete s;
@@ -431,6 +637,12 @@ extern "C" int sur_create(const sur_cfg_t *cfg, const sim_opts_t *opts, sur_t **
       return bail(sfail(s, SIM_ECUDA, cudaGetErrorString(e)));
     s->own_stream = true;
   }
+  for (int k = 0; k < sur_t::SIDES && e == cudaSuccess; k++)
+    if ((e = cudaStreamCreateWithFlags(&s->side[k], cudaStreamNonBlocking)) == cudaSuccess)
+      e = cudaEventCreateWithFlags(&s->done[k], cudaEventDisableTiming);
+  for (int k = 0; k < sur_t::MAX_READY && e == cudaSuccess; k++)
+    e = cudaEventCreateWithFlags(&s->ready[k], cudaEventDisableTiming);
+  if (e != cudaSuccess) return bail(sfail(s, SIM_ECUDA, cudaGetErrorString(e)));
   layout(s);
   const long long P = s->nparam;
   int rc;
@@ -453,15 +665,21 @@ extern "C" int sur_create(const sur_cfg_t *cfg, const sim_opts_t *opts, sur_t **
   zmax = std::max(zmax, amax);
   s->pre.resize(an.size());
   s->act.resize(an.size());
+  s->gz.resize(an.size());
+  s->gz16.resize(an.size());
   for (size_t l = 0; l < an.size(); l++) {
     if ((rc = salloc(s, &s->pre[l], an[l] * 4)) || (rc = salloc(s, &s->act[l], an[l] * 2))) return bail(rc);
+    // a convolution's dZ has two values per output (four taps, half as many inputs)
+    if (l > 0 && ((rc = salloc(s, &s->gz[l], an[l] * 4)) || (rc = salloc(s, &s->gz16[l], an[l] * (l > 3 ? 4 : 2)))))
+      return bail(rc);
   }
   if ((rc = salloc(s, &s->z, zmax * 4)) || (rc = salloc(s, &s->y, (long long)B * Lf * cfg->out_ch * 4)) ||
       (rc = salloc(s, &s->dy, (long long)B * Lf * cfg->out_ch * 4)) || (rc = salloc(s, &s->da, zmax * 4)) ||
-      (rc = salloc(s, &s->dz, zmax * 4)) || (rc = salloc(s, &s->dz16, zmax * 2)) ||
-      (rc = salloc(s, &s->dy16, zmax * 2)) || (rc = salloc(s, &s->part, 4096LL * 4096 * 4)) ||
-      (rc = salloc(s, &s->lossp, 4096 * 4)) || (rc = salloc(s, &s->xb, (long long)B * cfg->in_dim * 4)) ||
-      (rc = salloc(s, &s->tb, (long long)B * Lf * cfg->out_ch * 4)) || (rc = salloc(s, &s->idx, B * 4)))
+      (rc = salloc(s, &s->dz, (long long)B * Lf * cfg->out_ch * 4)) ||
+      (rc = salloc(s, &s->dy16, (long long)B * Lf * cfg->out_ch * 2)) ||
+      (rc = salloc(s, &s->part, (long long)COLSUM_PARTS * COLSUM_PARTS * 4)) ||
+      (rc = salloc(s, &s->lossp, LOSS_PARTS * 4)) || (rc = salloc(s, &s->xb, (long long)B * cfg->in_dim * 4)) ||
+      (rc = salloc(s, &s->tb, (long long)B * Lf * cfg->out_ch * 4)))
     return bail(rc);
   // initial weights: uniform +-sqrt(6 / (fan_in + fan_out)) from SplitMix64, biases 0
   std::vector<float> w(P, 0.f);
@@ -498,13 +716,12 @@ static float *Wp(sur_t *s, int slot) { return s->w + s->off[slot]; }
 static __nv_bfloat16 *W16(sur_t *s, int slot) { return s->w16 + s->off[slot]; }
 static float *Gp(sur_t *s, int slot) { return s->g + s->off[slot]; }
 
-static cudaError_t colsum(sur_t *s, const float *X, long long rows, int N, float *out) {
+static cudaError_t colsum(const float *X, long long rows, int N, float *out, float *part, cudaStream_t st) {
   const int chunk = 256;
-  const int parts = (int)std::min<long long>((rows + chunk - 1) / chunk, 4096);
+  const int parts = (int)std::min<long long>((rows + chunk - 1) / chunk, COLSUM_PARTS);
   const int ch = (int)((rows + parts - 1) / parts);
-  dim3 g1((N + 127) / 128, parts);
-  k_colsum_partial<<<g1, 128, 0, s->stream>>>(X, rows, N, ch, s->part);
-  k_colsum_final<<<(N + 127) / 128, 128, 0, s->stream>>>(s->part, parts, N, out);
+  k_colsum_partial<<<(int)(((long long)N * parts + 127) / 128), 128, 0, st>>>(X, rows, N, ch, parts, part);
+  k_colsum_final<<<(N + 31) / 32, 32, 0, st>>>(part, parts, N, out);
   return cudaGetLastError();
 }
 
@@ -517,7 +734,7 @@ static cudaError_t forward(sur_t *s, int n) {
   const int dims[4] = {c.in_dim, c.h1, c.h2, c.l0 * c.chans[0]};
   for (int l = 0; l < 3; l++) {
     if ((e = gemm(false, false, n, dims[l + 1], dims[l], s->act[l], dims[l], W16(s, 2 * l), dims[l + 1], s->z,
-                  dims[l + 1], 1.f, 0.f, st)) != cudaSuccess)
+                  dims[l + 1], st)) != cudaSuccess)
       return e;
     k_bias_gelu<<<egrid((long long)n * dims[l + 1]), 256, 0, st>>>(s->z, Wp(s, 2 * l + 1), n, dims[l + 1],
                                                                      s->pre[l + 1], s->act[l + 1]);
@@ -526,7 +743,7 @@ static cudaError_t forward(sur_t *s, int n) {
     const int Lin = c.l0 << l, Cin = c.chans[l], Cout = c.chans[l + 1];
     const long long rows = (long long)n * Lin;
     if ((e = gemm(false, false, (int)rows, Cout * 4, Cin, s->act[3 + l], Cin, W16(s, 6 + 2 * l), Cout * 4, s->z,
-                  Cout * 4, 1.f, 0.f, st)) != cudaSuccess)
+                  Cout * 4, st)) != cudaSuccess)
       return e;
     k_col2im<<<egrid(rows * 2 * Cout), 256, 0, st>>>(s->z, Wp(s, 7 + 2 * l), n, Lin, Cout, s->pre[4 + l],
                                                       s->act[4 + l]);
@@ -534,66 +751,75 @@ static cudaError_t forward(sur_t *s, int n) {
   const int Lf = L_out(s), Cl = c.chans[c.n_up];
   const long long rows = (long long)n * Lf;
   if ((e = gemm(false, false, (int)rows, c.out_ch, Cl, s->act[3 + c.n_up], Cl, W16(s, 6 + 2 * c.n_up), c.out_ch,
-                s->z, c.out_ch, 1.f, 0.f, st)) != cudaSuccess)
+                s->z, c.out_ch, st)) != cudaSuccess)
     return e;
   k_bias<<<egrid(rows * c.out_ch), 256, 0, st>>>(s->z, Wp(s, 7 + 2 * c.n_up), rows, c.out_ch, s->y);
   return cudaGetLastError();
 }
 
-// loss (host value) and gradient into s->g for the targets in s->tb
-static cudaError_t backward(sur_t *s, int n, float *loss_out) {
+// Gradient into s->g and the loss kernel's LOSS_PARTS partial sums into lossp
+// (device), for the targets in s->tb; the handle's stream ends behind all of it.
+static cudaError_t backward(sur_t *s, int n, float *lossp) {
   const sur_cfg_t &c = s->cfg;
   cudaStream_t st = s->stream;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   const int Lf = L_out(s), Cl = c.chans[c.n_up];
   const long long rows = (long long)n * Lf, count = rows * c.out_ch;
-  const int lblocks = 1024;
-  k_mse<<<lblocks, 256, 0, st>>>(s->y, s->tb, n, Lf, c.out_ch, 1.f / (float)count, 1.f / s->y_scale, s->dy, s->lossp);
-  if (loss_out) {
-    std::vector<float> lp(lblocks);
-    if ((e = cudaMemcpyAsync(lp.data(), s->lossp, lblocks * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    double acc = 0;
-    for (float x : lp) acc += x;
-    *loss_out = (float)(acc / (double)count);
-  }
+  int nready = 0;
+  // weight and bias gradient of one layer, operands just enqueued on st:
+  // dW[M x N] = A^T D over K rows, db = column sums of d (drows x N2)
+  auto grads = [&](int side, int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *D, float *dW,
+                   const float *d, long long drows, int N2, float *db) {
+    cudaEvent_t r = s->ready[nready++];
+    if ((e = cudaEventRecord(r, st)) != cudaSuccess) return e;
+    for (int k : {0, side})
+      if ((e = cudaStreamWaitEvent(s->side[k], r, 0)) != cudaSuccess) return e;
+    if ((e = colsum(d, drows, N2, db, s->part, s->side[0])) != cudaSuccess) return e;
+    return e = gemm_grad(M, N, K, A, M, D, N, dW, s->side[side]);
+  };
+  // data gradient: s->da = D W^T
+  auto data = [&](int M, int N, int K, const __nv_bfloat16 *D, const __nv_bfloat16 *W) {
+    return e = gemm(false, true, M, N, K, D, K, W, K, s->da, N, st);
+  };
+  k_mse<<<LOSS_PARTS, 256, 0, st>>>(s->y, s->tb, n, Lf, c.out_ch, 1.f / (float)count, 1.f / s->y_scale, s->dy, s->dy16,
+                                    lossp);
   // final 1x1 layer
-  k_to_bf16<<<egrid(count), 256, 0, st>>>(s->dy, count, s->dy16);
-  if ((e = gemm(true, false, Cl, c.out_ch, (int)rows, s->act[3 + c.n_up], Cl, s->dy16, c.out_ch,
-                Gp(s, 6 + 2 * c.n_up), c.out_ch, 1.f, 0.f, st)) != cudaSuccess)
+  if (grads(1, Cl, c.out_ch, (int)rows, s->act[3 + c.n_up], s->dy16, Gp(s, 6 + 2 * c.n_up), s->dy, rows, c.out_ch,
+            Gp(s, 7 + 2 * c.n_up)) != cudaSuccess)
     return e;
-  if ((e = colsum(s, s->dy, rows, c.out_ch, Gp(s, 7 + 2 * c.n_up))) != cudaSuccess) return e;
-  if ((e = gemm(false, true, (int)rows, Cl, c.out_ch, s->dy16, c.out_ch, W16(s, 6 + 2 * c.n_up), c.out_ch, s->da, Cl,
-                1.f, 0.f, st)) != cudaSuccess)
-    return e;
+  if (data((int)rows, Cl, c.out_ch, s->dy16, W16(s, 6 + 2 * c.n_up)) != cudaSuccess) return e;
   // transposed convolutions, last to first
   for (int l = c.n_up - 1; l >= 0; l--) {
     const int Lin = c.l0 << l, Cin = c.chans[l], Cout = c.chans[l + 1];
-    const long long orow = (long long)n * 2 * Lin, irow = (long long)n * Lin;
-    k_gelu_bwd<<<egrid(orow * Cout), 256, 0, st>>>(s->da, s->pre[4 + l], orow * Cout, s->dz, nullptr);
-    if ((e = colsum(s, s->dz, orow, Cout, Gp(s, 7 + 2 * l))) != cudaSuccess) return e;
-    k_im2col<<<egrid(irow * Cout * 4), 256, 0, st>>>(s->dz, n, Lin, Cout, s->dz16);
-    if ((e = gemm(true, false, Cin, Cout * 4, (int)irow, s->act[3 + l], Cin, s->dz16, Cout * 4, Gp(s, 6 + 2 * l),
-                  Cout * 4, 1.f, 0.f, st)) != cudaSuccess)
+    const long long irow = (long long)n * Lin;
+    k_conv_bwd<<<egrid(irow * Cout), 256, 0, st>>>(s->da, s->pre[4 + l], n, Lin, Cout, s->gz[4 + l], s->gz16[4 + l]);
+    if (grads(2, Cin, Cout * 4, (int)irow, s->act[3 + l], s->gz16[4 + l], Gp(s, 6 + 2 * l), s->gz[4 + l], 2 * irow,
+              Cout, Gp(s, 7 + 2 * l)) != cudaSuccess)
       return e;
-    if ((e = gemm(false, true, (int)irow, Cin, Cout * 4, s->dz16, Cout * 4, W16(s, 6 + 2 * l), Cout * 4, s->da, Cin,
-                  1.f, 0.f, st)) != cudaSuccess)
-      return e;
+    if (data((int)irow, Cin, Cout * 4, s->gz16[4 + l], W16(s, 6 + 2 * l)) != cudaSuccess) return e;
   }
   // dense layers 3, 2, 1
   const int dims[4] = {c.in_dim, c.h1, c.h2, c.l0 * c.chans[0]};
   for (int l = 2; l >= 0; l--) {
     const long long nel = (long long)n * dims[l + 1];
-    k_gelu_bwd<<<egrid(nel), 256, 0, st>>>(s->da, s->pre[l + 1], nel, s->dz, s->dz16);
-    if ((e = colsum(s, s->dz, n, dims[l + 1], Gp(s, 2 * l + 1))) != cudaSuccess) return e;
-    if ((e = gemm(true, false, dims[l], dims[l + 1], n, s->act[l], dims[l], s->dz16, dims[l + 1], Gp(s, 2 * l),
-                  dims[l + 1], 1.f, 0.f, st)) != cudaSuccess)
+    k_gelu_bwd<<<egrid(nel), 256, 0, st>>>(s->da, s->pre[l + 1], nel, s->gz[l + 1], s->gz16[l + 1]);
+    if (grads(2, dims[l], dims[l + 1], n, s->act[l], s->gz16[l + 1], Gp(s, 2 * l), s->gz[l + 1], n, dims[l + 1],
+              Gp(s, 2 * l + 1)) != cudaSuccess)
       return e;
-    if (l > 0 && (e = gemm(false, true, n, dims[l], dims[l + 1], s->dz16, dims[l + 1], W16(s, 2 * l), dims[l + 1],
-                           s->da, dims[l], 1.f, 0.f, st)) != cudaSuccess)
-      return e;
+    if (l > 0 && data(n, dims[l], dims[l + 1], s->gz16[l + 1], W16(s, 2 * l)) != cudaSuccess) return e;
+  }
+  for (int k = 0; k < sur_t::SIDES; k++) {
+    if ((e = cudaEventRecord(s->done[k], s->side[k])) != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(st, s->done[k], 0)) != cudaSuccess) return e;
   }
   return cudaGetLastError();
+}
+
+// the loss from the partial sums of a minibatch of n samples
+static float loss_of(const sur_t *s, const float *parts, int n) {
+  double acc = 0;
+  for (int q = 0; q < LOSS_PARTS; q++) acc += parts[q];
+  return (float)(acc / ((double)n * L_out(s) * s->cfg.out_ch));
 }
 
 extern "C" int sur_param_count(const sur_t *s, long long *n) {
@@ -698,12 +924,13 @@ extern "C" int sur_loss_grad(sur_t *s, const float *X, const float *Y, int n, fl
   SCK(s, cudaMemcpyAsync(s->xb, X, (size_t)n * c.in_dim * 4, cudaMemcpyHostToDevice, s->stream));
   SCK(s, cudaMemcpyAsync(s->tb, Y, (size_t)n * Lf * c.out_ch * 4, cudaMemcpyHostToDevice, s->stream));
   SCK(s, forward(s, n));
-  float l = 0.f;
-  SCK(s, backward(s, n, &l));
-  if (loss) *loss = l;
+  SCK(s, backward(s, n, s->lossp));
+  std::vector<float> lp(LOSS_PARTS);
+  SCK(s, cudaMemcpyAsync(lp.data(), s->lossp, LOSS_PARTS * 4, cudaMemcpyDeviceToHost, s->stream));
   // the gradient kernels run on the handle's (non-blocking) stream: copy on it and wait
   if (grad) SCK(s, cudaMemcpyAsync(grad, s->g, s->nparam * 4, cudaMemcpyDeviceToHost, s->stream));
   SCK(s, cudaStreamSynchronize(s->stream));
+  if (loss) *loss = loss_of(s, lp.data(), n);
   return tc_status(s);
 }
 
@@ -715,13 +942,23 @@ extern "C" int sur_train(sur_t *s, const float *X, const float *Y, int n, int ep
   const sur_cfg_t &c = s->cfg;
   const int Lf = L_out(s);
   const long long xrow = c.in_dim, yrow = (long long)Lf * c.out_ch;
-  float *dX = nullptr, *dY = nullptr;
-  SCK(s, cudaMalloc(&dX, (size_t)n * xrow * 4));
-  cudaError_t e = cudaMalloc(&dY, (size_t)n * yrow * 4);
+  const int per_epoch = (n + batch - 1) / batch;
+  // the data, the epoch's order and every minibatch's loss partials stay on
+  // the device, so that no minibatch waits for the host; the losses are read
+  // once per epoch
+  float *dX = nullptr, *dY = nullptr, *dL = nullptr;
+  int *dI = nullptr;
+  cudaError_t e = cudaMalloc(&dX, (size_t)n * xrow * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&dY, (size_t)n * yrow * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&dL, (size_t)per_epoch * LOSS_PARTS * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&dI, (size_t)n * 4);
   if (e != cudaSuccess) {
     cudaFree(dX);
+    cudaFree(dY);
+    cudaFree(dL);
     return sfail(s, SIM_ENOMEM, cudaGetErrorString(e));
   }
+  std::vector<float> lp((size_t)per_epoch * LOSS_PARTS);
   e = cudaMemcpyAsync(dX, X, (size_t)n * xrow * 4, cudaMemcpyHostToDevice, s->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dY, Y, (size_t)n * yrow * 4, cudaMemcpyHostToDevice, s->stream);
   std::vector<int> perm(n);
@@ -738,19 +975,13 @@ extern "C" int sur_train(sur_t *s, const float *X, const float *Y, int n, int ep
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   for (int ep = 0; ep < epochs && e == cudaSuccess; ep++) {
     for (int q = n - 1; q > 0; q--) std::swap(perm[q], perm[rnd() % (uint64_t)(q + 1)]);
-    double lsum = 0;
-    int nb_count = 0;
+    if ((e = cudaMemcpyAsync(dI, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess) break;
     for (int b0 = 0; b0 < n && e == cudaSuccess; b0 += batch) {
       const int nb = std::min(batch, n - b0);
-      e = cudaMemcpyAsync(s->idx, perm.data() + b0, nb * 4, cudaMemcpyHostToDevice, s->stream);
-      if (e != cudaSuccess) break;
-      k_gather<<<egrid(nb * xrow), 256, 0, s->stream>>>(dX, s->idx, nb, xrow, s->xb);
-      k_gather<<<egrid(nb * yrow), 256, 0, s->stream>>>(dY, s->idx, nb, yrow, s->tb);
+      k_gather<<<egrid(nb * xrow), 256, 0, s->stream>>>(dX, dI + b0, nb, xrow, s->xb);
+      k_gather<<<egrid(nb * yrow), 256, 0, s->stream>>>(dY, dI + b0, nb, yrow, s->tb);
       if ((e = forward(s, nb)) != cudaSuccess) break;
-      float l = 0.f;
-      if ((e = backward(s, nb, &l)) != cudaSuccess) break;
-      lsum += l;
-      nb_count++;
+      if ((e = backward(s, nb, dL + (size_t)(b0 / batch) * LOSS_PARTS)) != cudaSuccess) break;
       // cosine learning-rate schedule over all steps
       const float lr_t = 0.5f * lr * (1.f + cosf(3.14159265f * (float)step / (float)std::max<long long>(1, steps_total)));
       s->adam_t++;
@@ -760,11 +991,18 @@ extern "C" int sur_train(sur_t *s, const float *X, const float *Y, int n, int ep
                                                        c2);
       e = cudaGetLastError();
     }
-    if (epoch_loss) epoch_loss[ep] = (float)(lsum / std::max(1, nb_count));
+    // the copy also keeps the host's order from being reshuffled before it is uploaded
+    if (e == cudaSuccess) e = cudaMemcpyAsync(lp.data(), dL, lp.size() * 4, cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    double lsum = 0;
+    for (int q = 0; q < per_epoch; q++) lsum += loss_of(s, lp.data() + (size_t)q * LOSS_PARTS, std::min(batch, n - q * batch));
+    if (epoch_loss) epoch_loss[ep] = (float)(lsum / per_epoch);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   cudaFree(dX);
   cudaFree(dY);
+  cudaFree(dL);
+  cudaFree(dI);
   if (e != cudaSuccess) return sfail(s, SIM_ECUDA, cudaGetErrorString(e));
   return tc_status(s);
 }
@@ -816,6 +1054,7 @@ extern "C" void sur_destroy(sur_t *s) {
   if (!s) return;
   cudaSetDevice(s->device);
   if (s->stream) cudaStreamSynchronize(s->stream);
+  release_side(s);
   for (void *p : s->allocs) cudaFree(p);
   if (s->own_stream) cudaStreamDestroy(s->stream);
   delete s;
@@ -841,7 +1080,7 @@ extern "C" int cw_gemm_bf16_path(int path, int trans_a, int trans_b, int M, int 
   if (e == cudaSuccess) e = cudaMemcpy(dA, A, na * 2, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(dB, B, nb * 2, cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
-    e = gemm_path(path, trans_a != 0, trans_b != 0, M, N, K, dA, lda, dB, ldb, dC, ldc, 1.f, 0.f, 0);
+    e = gemm_path(path, trans_a != 0, trans_b != 0, M, N, K, dA, lda, dB, ldb, dC, ldc, 0);
   if (e == cudaSuccess) e = cudaMemcpy(C, dC, nc * 4, cudaMemcpyDeviceToHost);
   int st = 0;
   if (e == cudaSuccess) e = gemm_tcgen05_status(&st, 0);

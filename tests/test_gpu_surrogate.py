@@ -187,3 +187,31 @@ def test_sensitivity_against_the_reference_network():
     print("sensitivity", sens.round(4), "reference", ref.round(4))
     assert np.all(ref > 0)
     assert np.all(np.abs(sens - ref) <= 0.05 * ref + 1e-3), (sens, ref)
+
+
+@pytest.mark.parametrize("n,l0,chans", [
+    (7, 20, (24, 40, 8)),   # K = 140, 280 below and 560 above the weight-gradient kernel's minimum, ragged tiles
+    (4, 64, (16, 8)),       # the last layer at K = 512 exactly, one tile
+    (3, 50, (64, 16, 8)),   # K = 600 over several column tiles
+    (5, 66, (12, 20)),      # channels that are no multiple of 8: rows are not 16-byte aligned
+])
+def test_weight_gradients_at_ragged_shapes(n, l0, chans):
+    """loss_grad on small odd networks against the FP64 reference with the
+    same rounding points, tensor by tensor (the bars of
+    test_forward_and_gradient_match_fp64_reference: BF16 operands, 2^-9
+    relative each, leave the cosine above 0.999)."""
+    from paper_2302_13907_gb300.binding import Surrogate
+    shp = R.shapes(h1=16, h2=24, c0=chans[0], l0=l0, chans=chans[1:])
+    rng = np.random.default_rng(n * 100 + l0)
+    X = rng.uniform(-1, 1, (n, 6)).astype(np.float32)
+    with Surrogate(max_batch=n, seed=2, h1=16, h2=24, l0=l0, chans=chans) as s:
+        thb = _bf16_theta(s.params(), shp)
+        T = rng.standard_normal((n, 8, l0 * 2 ** (len(chans) - 1))).astype(np.float32)
+        _, g = s.loss_grad(X, T)
+    _, gq = R.loss_and_grad(thb, X.astype(np.float64), T.astype(np.float64), shp, c0=chans[0], l0=l0, q=bf16_round)
+    assert cosine(g, gq) >= 0.999
+    o = 0
+    for name, sh in shp:
+        k = int(np.prod(sh))
+        assert cosine(g[o:o + k], gq[o:o + k]) >= 0.99, name
+        o += k
