@@ -338,8 +338,7 @@ cudaError_t launch_sweep(int storage, int code, const KParams &p, int *vdone, in
 // BF16 GEMM on the tcgen05 tensor cores (gemm_tc.cu); status bit 0: a
 // bounded wait gave up (read and cleared by gemm_tcgen05_status)
 cudaError_t gemm_tcgen05(bool ta, bool tb, int M, int N, int K, const __nv_bfloat16 *A, int lda,
-                         const __nv_bfloat16 *B, int ldb, float *C, int ldc, float alpha, float beta,
-                         cudaStream_t s);
+                         const __nv_bfloat16 *B, int ldb, float *C, int ldc, cudaStream_t s);
 cudaError_t gemm_tcgen05_status(int *out, cudaStream_t s);
 int march_box_x(int storage);
 int march_box_id();

@@ -178,7 +178,7 @@ static cudaError_t gemm_mma(bool ta, bool tb, int M, int N, int K, const __nv_bf
 static cudaError_t gemm_path(int path, bool ta, bool tb, int M, int N, int K, const __nv_bfloat16 *A, int lda,
                              const __nv_bfloat16 *B, int ldb, float *C, int ldc, cudaStream_t s) {
   const bool tc = path == 2 || (path == 0 && M >= 128);
-  return tc ? gemm_tcgen05(ta, tb, M, N, K, A, lda, B, ldb, C, ldc, 1.f, 0.f, s)
+  return tc ? gemm_tcgen05(ta, tb, M, N, K, A, lda, B, ldb, C, ldc, s)
             : gemm_mma(ta, tb, M, N, K, A, lda, B, ldb, C, ldc, s);
 }
 
