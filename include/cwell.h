@@ -274,18 +274,18 @@ size_t sim_device_bytes(const sim_t *h);
  * the split kernels, 2000 + b for their load-first variant (four z cells per
  * thread) compiled for b resident blocks per SM (b = 3, 4, 5; blocks walk theta
  * fastest), 2010 + b for the same with the blocks walking z fastest (b = 3, 4),
- * 2100 + b for two z cells per thread (b = 6, 8), 2200 + 10 c + b for interior /
- * edge split launches (a kernel with the interior body only on the tiles away
- * from every PML and end, compiled for b blocks per SM, and the general kernel
- * on the rest; interior four cells per thread, b = 4, 5, with edge c = 0 (four
- * cells, 4 blocks/SM), 2 (two, 4), 3 (two, 6), 4 (four, 3); interior two
- * cells, b = 6, 8, with edge c = 1 (two, 6) or 5 (two, 4); c = 6, 7 as 2, 4
- * with a persistent interior kernel prefetching its next tile into L2; c = 8
- * as 4 and c = 9 as 6, each with the edge tiles walked by a persistent
- * prefetching kernel); 2300 + 10 c + b for a three-way split (interior; the
- * radial-PML rows' interior z tiles with a body for interior z; the z ends),
- * interior b = 5 plain or 4 prefetching, c = 0 to 3 the radial / end kernels'
- * cells per thread and blocks per SM;
+ * 2100 + b for two z cells per thread (b = 6, 8), 2200 + 10 c + b for the
+ * interior / edge split (the cells away from every PML and end with a lean body,
+ * compiled for b blocks per SM; the radial-PML rows and the z ends with their
+ * own): interior four cells per thread, b = 4, 5, with edge c = 0 (four cells, 4
+ * blocks/SM), 2 (two cells, both in one launch), 3 (two, 6), 4 (four, 3);
+ * interior two cells, b = 6, 8, with edge c = 1 (two, 6) or 5 (two; b = 6 in one
+ * launch, b = 8 edge for 4 blocks/SM); c = 6, 7: edge (two, 4), (four, 3) with a
+ * persistent interior kernel prefetching its next tile into L2; c = 8 as 4 and
+ * c = 9 as 6, each with the radial tiles walked the same way; 2300 + 10 c + b
+ * for a three-way split (interior; radial-PML rows; z ends), interior b = 5
+ * plain or 4 prefetching, c = 0 to 3 the radial / end kernels' cells per thread
+ * and blocks per SM;
  * v * 10000 + s (a pair code) for the velocity kernel of split code v with the
  * stress kernel of split code s; 3000 + 100 m + 10 e + b for the single-pass
  * sweep kernel (kernel = SIM_KERNEL_SWEEP: four z cells per thread, b resident
@@ -335,10 +335,8 @@ const char *sim_error_string(int code);
  * receivers; shapes may differ between cases); opts is shared (storage,
  * stream, device, mem_cap applied to the batch total, graph_chunk,
  * max_steps; opts.kernel is ignored).  Cases of fewer than 4 Mi cells share
- * one interior and one edge launch per half step of the load-first split
- * bodies, driven by blocks that walk a work list of (case, theta, r tile, z
- * tile) items; the number of blocks is chosen by timing candidates at create
- * time.  A larger case fills the GPU alone and runs its own split launches
+ * one launch per half step of the load-first split bodies, one block per tile
+ * of a case.  A larger case fills the GPU alone and runs its own split launches
  * with the code its tuner picks (as sim_create with kernel SIM_KERNEL_SPLIT);
  * those cases are spread over 1, 2 or 4 parallel streams (branches of the
  * captured graph, the count timed at create time), so that one case's launch
@@ -364,7 +362,7 @@ int simb_sync(simb_t *b);
 int simb_traces(simb_t *b, int which, float *out, size_t cap, int *n_rec, int *n_steps);
 int simb_read_field(simb_t *b, int which, int field, float *out, size_t n);
 
-/* Number of cases, work items of the shared launches, persistent blocks per shared launch. */
+/* Number of cases, work items (tiles) and blocks of one shared launch. */
 int simb_config(const simb_t *b, int *n_cases, long long *work_items, int *grid_blocks);
 /* Cases on their own launches and the parallel streams they run on. */
 int simb_layout(const simb_t *b, int *own_cases, int *branches);
@@ -394,10 +392,10 @@ const char *simb_last_error(const simb_t *b);
  * storage; any source kind, placed on the nodes of the zone that holds it
  * (the transverse force off the axis and the torsion ring not on a zone's
  * first row, SIM_EUNSUPPORTED).  Every zone runs the split kernels, velocity
- * code 2285 and stress code 2324 (largest zone of at least 8 Mi cells; the
- * zones of a half then run on parallel streams) or 2294 (smaller grids, zones
- * one after another) unless opts.tile names a 22xx / 23xx split code or pair
- * code (SIM_EINVAL otherwise).
+ * code 2285 and stress code 2334 (largest zone of at least 8 Mi cells; the
+ * zones of a half then run on parallel streams); on smaller grids all zones of
+ * a half share one launch.  opts.tile may name a 22xx / 23xx split code or pair
+ * code instead (SIM_EINVAL otherwise; small grids then run zone after zone).
  * Ownership and errors as sim_create; simr_last_error(NULL) after a failed create.
  * ------------------------------------------------------------------------ */
 typedef struct {

@@ -18,10 +18,10 @@ struct simb_s {
   bool own_stream = false;
   std::vector<sim_t *> cases;
   std::vector<KParams> kp;        // the cases' kernel parameters (host: they travel as kernel parameters)
-  std::vector<int> shared, own;   // cases in the shared persistent launches / on their own tuned launches
+  std::vector<int> shared, own;   // cases in the shared launches / on their own tuned launches
   RParams *d_rp = nullptr;
-  long long total = 0;  // bound on the items of one work list of the shared cases
-  int grid = 0, graph_chunk = 64, steps_done = 0;
+  long long total = 0;  // blocks of the shared cases in one half step
+  int graph_chunk = 64, steps_done = 0;
   // parallel streams for the own-launch cases: case own[q] runs on branch[q % nbranch]
   static constexpr int MAX_BRANCH = 4;
   cudaStream_t branch[MAX_BRANCH] = {};
@@ -59,7 +59,7 @@ static void brelease(simb_t *b) {
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
 }
 
-// Small cases share the persistent batched launches (one case cannot fill the
+// Small cases share the batched launches (one case cannot fill the
 // GPU); a case of at least OWN_CELLS cells fills it alone and runs its own
 // split launches with the code its tuner chose (the prefetching kernels), in
 // the same stream and graph.
@@ -79,7 +79,7 @@ static cudaError_t batch_step(simb_t *b, const KParams *cases) {
     for (int k = 0; k < nb && e == cudaSuccess; k++) e = cudaStreamWaitEvent(b->branch[k], b->fork, 0);
   }
   for (int half = 1; half <= 2 && e == cudaSuccess; half++) {
-    if (!sh.empty()) e = launch_batch_split(b->storage, half == 1, sh.data(), (int)sh.size(), b->grid, b->stream);
+    if (!sh.empty()) e = launch_batch_split(b->storage, half == 1, sh.data(), (int)sh.size(), b->stream);
     for (size_t q = 0; q < b->own.size() && e == cudaSuccess; q++)
       e = sim_split_halves(b->cases[b->own[q]], cases[b->own[q]], stream_of(q), half);
   }
@@ -91,11 +91,10 @@ static cudaError_t batch_step(simb_t *b, const KParams *cases) {
   return e;
 }
 
-// time persistent grids of several sizes (and one block per item) on the
+// branches of the own-launch cases: 1, 2 or 4 parallel streams, timed on the
 // still-zero state with every source disabled; keep the fastest
-static int tune_grid(simb_t *b) {
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
+static int tune_branches(simb_t *b) {
+  if (b->own.size() < 2 || b->fixed_branches) return SIM_OK;
   const int n = (int)b->cases.size();
   std::vector<KParams> dry(n);
   for (int c = 0; c < n; c++) {
@@ -106,13 +105,11 @@ static int tune_grid(simb_t *b) {
   cudaEvent_t t0, t1;
   cudaEventCreate(&t0);
   cudaEventCreate(&t1);
-  const long long cand[5] = {(long long)sms * 6, (long long)sms * 12, (long long)sms * 24, (long long)sms * 48,
-                             b->total};
+  int pick = 1;
   float best = INFINITY;
-  int pick = (int)std::min<long long>(b->total, (long long)sms * 12);
-  for (long long g : cand) {
-    if (e != cudaSuccess) break;
-    b->grid = (int)std::max<long long>(1, std::min<long long>(g, std::min<long long>(b->total, 1LL << 30)));
+  for (int nb : {1, 2, 4}) {
+    if (nb > (int)b->own.size() || e != cudaSuccess) break;
+    b->nbranch = nb;
     e = batch_step(b, dry.data());
     cudaEventRecord(t0, b->stream);
     for (int w = 0; w < 3 && e == cudaSuccess; w++) e = batch_step(b, dry.data());
@@ -122,31 +119,10 @@ static int tune_grid(simb_t *b) {
     cudaEventElapsedTime(&ms, t0, t1);
     if (e == cudaSuccess && ms < best) {
       best = ms;
-      pick = b->grid;
+      pick = nb;
     }
   }
-  b->grid = pick;
-  // branches of the own-launch cases: 1, 2 or 4 parallel streams
-  int pick_b = 1;
-  if (e == cudaSuccess && b->own.size() > 1 && !b->fixed_branches) {
-    float best_b = INFINITY;
-    for (int nb : {1, 2, 4}) {
-      if (nb > (int)b->own.size() || e != cudaSuccess) break;
-      b->nbranch = nb;
-      e = batch_step(b, dry.data());
-      cudaEventRecord(t0, b->stream);
-      for (int w = 0; w < 3 && e == cudaSuccess; w++) e = batch_step(b, dry.data());
-      cudaEventRecord(t1, b->stream);
-      if (e == cudaSuccess) e = cudaEventSynchronize(t1);
-      float ms = 0;
-      cudaEventElapsedTime(&ms, t0, t1);
-      if (e == cudaSuccess && ms < best_b) {
-        best_b = ms;
-        pick_b = nb;
-      }
-    }
-    b->nbranch = pick_b;
-  }
+  b->nbranch = pick;
   cudaEventDestroy(t0);
   cudaEventDestroy(t1);
   if (e != cudaSuccess) return bcuda(b, e, "batch autotune");
@@ -198,7 +174,7 @@ extern "C" int simb_create(int n, const sim_grid_t *grids, const sim_medium_t *m
     if ((e = cudaStreamCreateWithFlags(&b->branch[k], cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming)) != cudaSuccess)
       return bail(bcuda(b, e, "batch branches"));
-  // opts.tile of a batch: 1 = every case in the shared persistent launches,
+  // opts.tile of a batch: 1 = every case in the shared launches,
   // -b (b = 1, 2, 4) = b branches for the own-launch cases; 0 = tuned
   const bool all_shared = opts->tile == 1;
   if (opts->tile < 0) {
@@ -223,10 +199,11 @@ extern "C" int simb_create(int n, const sim_grid_t *grids, const sim_medium_t *m
     if (rc) return bail(bfail(b, rc, "case " + std::to_string(c) + ": " + sim_last_error(nullptr)));
     b->cases.push_back(h);
     used += sim_device_bytes(h);
-    const long long items = split_items(grids[c].nth, grids[c].nr + grids[c].pml_r, grids[c].nz + 2 * grids[c].pml_z);
-    if (!own && items > 0x7fffffffLL)
+    if (own) continue;
+    const long long blocks = batch_blocks(h->kp);
+    if (blocks > 0x7fffffffLL)
       return bail(bfail(b, SIM_EINVAL, "case " + std::to_string(c) + ": more work items than a 32-bit index holds"));
-    if (!own) b->total += items;  // work items of the shared launches
+    b->total += blocks;
   }
   b->kp.resize(n);
   std::vector<RParams> rp(n);
@@ -240,7 +217,7 @@ extern "C" int simb_create(int n, const sim_grid_t *grids, const sim_medium_t *m
   }
   if ((e = cudaMemcpy(b->d_rp, rp.data(), n * sizeof(RParams), cudaMemcpyHostToDevice)) != cudaSuccess)
     return bail(bcuda(b, e, "upload batch tables"));
-  int rc = tune_grid(b);
+  int rc = tune_branches(b);
   if (rc) return bail(rc);
   *out = b;
   return SIM_OK;
@@ -314,7 +291,7 @@ extern "C" int simb_config(const simb_t *b, int *n_cases, long long *work_items,
   if (!b) return SIM_EINVAL;
   if (n_cases) *n_cases = (int)b->cases.size();
   if (work_items) *work_items = b->total;
-  if (grid_blocks) *grid_blocks = b->grid;
+  if (grid_blocks) *grid_blocks = (int)std::min<long long>(std::max<long long>(1, b->total), 0x7fffffff);
   return SIM_OK;
 }
 

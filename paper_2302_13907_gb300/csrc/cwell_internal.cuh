@@ -226,13 +226,12 @@ cudaError_t launch_receivers(int storage, const RParams &p, cudaStream_t s);
 cudaError_t launch_inject(int storage, const IParams &p, cudaStream_t s);
 cudaError_t launch_fused(int storage, int rt, const FusedMaps &maps, const FusedParams &fp, cudaStream_t s);
 size_t fused_smem_bytes(int storage, int rt);
-// upper bound on the work items of one case in either batched work list
-long long split_items(int nth, int NR, int NZ);
-// batched load-first kernels (interior and edge launches per half step): cases
-// is a host array, launched in chunks of BATCH_MAX cases whose parameters
-// travel in the kernel's parameter space; grid = persistent blocks per launch
+// batched load-first kernel (one launch per half step): cases is a host array,
+// launched in chunks of BATCH_MAX cases whose parameters travel in the kernel's
+// parameter space; batch_blocks: blocks one case takes in a launch
 constexpr int BATCH_MAX = 64;
-cudaError_t launch_batch_split(int storage, bool vel, const KParams *cases, int n_cases, int grid, cudaStream_t s);
+long long batch_blocks(const KParams &p);
+cudaError_t launch_batch_split(int storage, bool vel, const KParams *cases, int n_cases, cudaStream_t s);
 cudaError_t launch_batch_receivers(int storage, const RParams *rp, int n_cases, cudaStream_t s);
 
 // Azimuthally refined grid: ghost rows filled from the neighbouring zone's
@@ -273,23 +272,23 @@ size_t march_smem_bytes(int storage, int code);
 // resident blocks per SM asked of the register allocator (b = 3, 4 or 5) and
 // block order o (0: theta fastest, 1: z fastest; b = 3 or 4 only); 2100 + b =
 // the two-cells-per-thread variant, theta fastest (b = 6 or 8); 2200 + 10 c + b
-// = interior / edge split launches (a lean-only interior kernel for b blocks per
-// SM, the general kernel on the PML and end tiles): c = 1: two cells per thread
+// = interior / edge split (a lean-only interior kernel for b blocks per SM;
+// radial-PML rows and z ends in an edge kernel): c = 1: two cells per thread
 // in both (b = 6 or 8; edge for 6 blocks per SM); otherwise four cells per
 // thread in the interior (b = 4 or 5) and an edge kernel with c = 0: four cells,
-// 4 blocks per SM; c = 2: two cells, 4 blocks; c = 3: two cells, 6 blocks;
-// c = 4: four cells, 3 blocks; c = 5: two cells in both (interior b = 6 or 8,
-// edge for 4 blocks per SM); c = 6 / 7: as c = 2 / 4 with a persistent
-// interior kernel that prefetches its next tile into L2; c = 8: plain
-// interior, edge (four cells, 3 blocks) walked by a persistent prefetching
-// kernel; c = 9: prefetching interior and prefetching edge (two cells, 4
-// blocks); 2300 + 10 c + b = three-way split (interior, radial-PML rows with a
-// body for interior z, z ends with the general body; persistent prefetching
-// kernels for the last two): interior b = 5 plain, 4 prefetching, and c = 0:
-// radial (four cells, 4 blocks per SM) + ends (four, 3); 1: (two, 5) + (two,
-// 4); 2: (two, 4) + (two, 4); 3: (four, 3) + (four, 3).  A pair code
-// v * 10000 + s runs the velocity kernel of split code v and the stress kernel
-// of split code s (the autotuner times the two apart).
+// 4 blocks per SM; c = 2: two cells, interior and edge in one launch for b
+// blocks per SM; c = 3: two cells, 6 blocks; c = 4: four cells, 3 blocks; c = 5:
+// two cells in both, b = 6: one launch for 5 blocks per SM, b = 8: interior for
+// 8, edge for 4; c = 6 / 7: two cells, 4 blocks / four cells, 3 blocks with a
+// persistent interior kernel that prefetches its next tile into L2; c = 8: plain
+// interior, edge (four cells, 3 blocks) whose radial tiles are walked with the
+// same prefetch; c = 9: prefetching interior and prefetching edge (two cells, 4
+// blocks); 2300 + 10 c + b = three-way split (interior, radial-PML rows, z ends;
+// the radial kernel persistent and prefetching): interior b = 5 plain, 4
+// prefetching, and c = 0: radial (four cells, 4 blocks per SM) + ends (four, 3);
+// 1: (two, 5) + (two, 4); 2: (two, 4) + (two, 4); 3: (four, 3) + (four, 3).  A
+// pair code v * 10000 + s runs the velocity kernel of split code v and the
+// stress kernel of split code s (the autotuner times the two apart).
 constexpr int SPLIT_CODE = 2000;
 inline bool is_split_single(int code) { return code >= 2000 && code < 3000; }
 inline bool is_split_pair(int code) {
@@ -298,14 +297,8 @@ inline bool is_split_pair(int code) {
 inline bool is_split_family(int code) { return is_split_single(code) || is_split_pair(code); }
 inline int split_vel_code(int code) { return code >= 10000 ? code / 10000 : code; }
 inline int split_str_code(int code) { return code >= 10000 ? code % 10000 : code; }
+inline bool is_sr_code(int code) { return code >= 2300 && code < 2400; }  // codes with the stochastic-rounding stores
 inline bool is_hoist(int code) { return code > 2000 && code < 3000; }
-inline int hoist_blocks(int code) { return code % 10; }
-inline bool hoist_split(int code) { return (code / 100) % 10 == 2 || (code / 100) % 10 == 3; }
-inline bool hoist_zfast(int code) { return !hoist_split(code) && (code / 10) % 10 == 1; }
-inline int hoist_cells_per_thread(int code) {
-  const int c = (code / 10) % 10;
-  return ((code / 100) % 10 == 1 || ((code / 100) % 10 == 2 && (c == 1 || c == 5))) ? 2 : 4;
-}
 // FP16 stochastic rounding of n device values with the given 13-bit dithers
 // (the rule of the FP16-SR stores), FP16 bit patterns out
 cudaError_t launch_watchdog(int storage, const WParams &p, int blocks, cudaStream_t s);

@@ -112,8 +112,8 @@ int cwell::validate_inputs(const sim_grid_t *g, const sim_medium_t *m, const sim
       return fail(nullptr, SIM_EUNSUPPORTED, "storage: stochastic rounding runs on the split and sweep kernels only");
     if (s->kind != 0)
       return fail(nullptr, SIM_EUNSUPPORTED, "storage: stochastic rounding with the volumetric source only");
-    if (o->tile != 0 && !(o->tile >= 2300 && o->tile < 2400) && !is_sweep(o->tile) &&
-        !(is_split_pair(o->tile) && split_vel_code(o->tile) / 100 == 23 && split_str_code(o->tile) / 100 == 23))
+    if (o->tile != 0 && !is_sr_code(o->tile) && !is_sweep(o->tile) &&
+        !(is_split_pair(o->tile) && is_sr_code(split_vel_code(o->tile)) && is_sr_code(split_str_code(o->tile))))
       return fail(nullptr, SIM_EUNSUPPORTED, "storage: stochastic rounding runs on the 23xx split and the sweep codes");
   }
   if (o->kernel < 0 || o->kernel > 5) return fail(nullptr, SIM_EINVAL, "opts: kernel must be 0 .. 5");
@@ -338,7 +338,7 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
     // a slab: the interior / edge split codes, whose kernels honour its z range
     if (h->slab && !(rt >= 2200 && rt < 2400)) continue;
     // stochastic rounding: the three-way split codes and the sweep kernel only
-    if (h->stencil_storage == SIM_STORAGE_F16_SR && !(rt >= 2300 && rt < 2400) && !is_sweep(rt)) continue;
+    if (h->stencil_storage == SIM_STORAGE_F16_SR && !is_sr_code(rt) && !is_sweep(rt)) continue;
     if (forced && rt != forced) continue;
     if (forced) {  // a tile asked for by the caller: check that it fits, time nothing
       const size_t need = is_split_family(rt) || is_sweep(rt) ? 1

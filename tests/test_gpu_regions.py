@@ -1,0 +1,47 @@
+"""Split half steps at the edges of their regions: where the lean z cells start
+or end inside a tile, on a tile, or in a sliver of one that goes to the z ends,
+and where the rows fill no whole tile."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2302_13907_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("tile", [2224, 2256, 2285, 2294, 2334])
+@pytest.mark.parametrize("nr,pml_r,nz,pml_z", [
+    (6, 1, 117, 2),     # lean cells 4 .. 116: one tile, cut at both ends
+    (5, 3, 146, 3),     # lean cells 4 .. 148: the second tile would hold 20, so the z ends take them
+    (7, 2, 60, 98),     # lean cells 100 .. 156: the first tile's 28 go to the z ends
+    (4, 4, 252, 4),     # rows and z cells fill whole tiles
+    (9, 1, 8, 5),       # no lean cell at all
+])
+def test_fields_at_region_edges(tile, nr, pml_r, nz, pml_z):
+    """Every field against the oracle, element by element (2e-5 of its maximum,
+    the bar of the split kernels' other element-wise tests)."""
+    from paper_2302_13907_gb300.binding import Simulation
+    g = W.Grid(nr=nr, nth=4, nz=nz, pml_r=pml_r, pml_z=pml_z, dr=0.004, dz=0.003)
+    rng = np.random.default_rng(nz)
+    mats = [W.FLUID, W.STEEL, W.CEMENT, W.ROCK]
+    cid = rng.integers(0, len(mats), size=g.shape).astype(np.uint16)
+    cid[:, 0, :] = 0
+    med = W.Medium(g, cid, *(np.array([m[q] for m in mats]) for q in range(3)))
+    sc = W.Scenario("edges", med, W.Source(r=0.009, theta=2.0, z=0.012, f0=60e3), W.on_axis_receivers([0.0]), steps=50)
+    o = oracle.Oracle(sc)
+    with Simulation(sc, kernel="split", tile=tile) as s:
+        for n in ("vr", "vp", "vz"):  # waves everywhere (v_r on the axis, v_z past the end are no unknowns)
+            v = 1e-7 * rng.standard_normal(g.shape).astype(np.float32)
+            if n == "vr":
+                v[:, 0] = 0
+            if n == "vz":
+                v[:, :, -1] = 0
+            s.set_field(n, v)
+            o.field(n)[...] = v
+        s.step(sc.steps)
+        o.step(sc.steps)
+        for n in oracle.FIELDS:
+            b = o.field(n)
+            assert np.abs(b).max() > 0, n
+            assert np.abs(s.field(n) - b).max() <= 2e-5 * np.abs(b).max(), n
