@@ -163,6 +163,8 @@ def launches_per_step(kind, tile):
     split half (23xx) three."""
     if kind in (2, 5):  # fused or sweep kernel + receivers
         return 2
+    if kind == 6:  # one-pass kernel, edge velocities, layer stresses, rim stresses, receivers
+        return 5
     if kind == 4:
         return 3
     per_half = {22: 2, 23: 3}  # interior + edge; interior + radial + ends
@@ -178,6 +180,8 @@ def kernel_label(kind, tile):
         return "march"
     if kind == 5:
         return f"sweep ({tile})"
+    if kind == 6:
+        return f"one-pass ({tile})"
     if tile >= 10000:
         return f"split (velocity {split_half_code(tile, True)}, stress {split_half_code(tile, False)})"
     return "split (load-first)" if tile > 2000 else "split"
@@ -596,6 +600,9 @@ def main():
         qd, per_cell = 0, b_fused
     elif kind == 5:  # one launch per step: both halves, every field read and written once
         names = [f"sweep_step:{tile}", "-", "receivers"]
+        qd, per_cell = 0, b_fused
+    elif kind == 6:  # both halves of the lean cells in one kernel, the edge cells' split halves beside it
+        names = [f"one_pass:{tile}", "edge_stresses", "receivers"]
         qd, per_cell = 0, b_fused
     else:
         names = ["march_step(velocity)", "march_step(stress)", "receivers"] if kind == 4 else \

@@ -70,6 +70,8 @@ extern "C" {
 #define SIM_KERNEL_MARCH 4     /* velocity and stress kernels marching theta over TMA-staged planes */
 #define SIM_KERNEL_SWEEP 5     /* one persistent launch per step sweeping z in chunks: both half-steps,
                                   each chunk's velocities and stresses reused from L2 */
+#define SIM_KERNEL_ONEPASS 6   /* reported by sim_config where AUTO chose the one-pass step (tile codes 4001 ..
+                                  4332); not a value of opts.kernel */
 
 /* Grid (Sec. 3): interior cell counts, PML widths in cells, steps in metres.
  * nth must be even and >= 4; nr >= 2; nz >= 2.  dt > 0 fixes the time step;
@@ -294,6 +296,12 @@ size_t sim_device_bytes(const sim_t *h);
  * m = 2, 3: chunks of 64 cells 2.5 chunks behind, m = 4, 5: chunks of 32
  * cells 2.5 and 2 chunks behind; m = 1, 3 add an L2 prefetch of each block's
  * next velocity item).
+ * 4000 + 100 m + d the one-pass step (kernel = AUTO, FP32, a second field set
+ * in memory, at least 4 rows and 32 z cells away from the PML, up to about 3500
+ * materials; SIM_EINVAL otherwise): both halves of the lean cells in one kernel,
+ * theta in d runs (1 .. nth, at most 32) per tile, m = 0, 2: one block per SM
+ * walks the tiles, 1, 3: one block per tile; the other cells with split bodies of
+ * two (m = 0, 1) or four (2, 3) cells per thread.
  * opts.tile accepts every code listed here. */
 int sim_config(const sim_t *h, int *kernel, int *tile_rows);
 

@@ -219,6 +219,26 @@ struct FusedParams {
   int *status;  // bit 1: a bounded wait gave up
 };
 
+// The set a step out of place writes (and whose velocities its stress half
+// reads); in place it is KParams.f.
+struct OutSet {
+  void *f[NF];
+};
+// One-pass step (stencil_pass.cu): k.f is read, out written; the launcher
+// fills the tiling.  status bit 1: a bounded wait gave up.
+struct PassParams {
+  KParams k;
+  OutSet out;
+  int *status;
+  int n_mat;
+  // point force: the v_r (or v_z) node (j, force_i, force_k) gains force_w[j] force_wav[step] (force_i < 0: none)
+  int force_i, force_k;
+  bool force_vz;
+  const float *force_w, *force_wav;
+  int r1, z0, z1;  // cells updated: rows [0, r1), z [z0, z1)
+  int ks0, nzt, tiles, tiles1, run1, run2, items1, items;
+};
+
 // launchers implemented in the .cu files (host side)
 // parts: 1 = velocity kernel, 2 = stress kernel, 3 = both (velocity first)
 cudaError_t launch_split(int storage, const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts = 3);
@@ -317,6 +337,23 @@ struct SideStream {
   cudaEvent_t fork, join;
 };
 void set_side_stream(const SideStream *ss);
+// one-pass step: tile code 4000 + 100 m + d, theta cut into d runs per tile;
+// m odd: one block per item, even: one block per SM walks them; m = 0, 1: the
+// split bodies on the rest of the cells take two cells per thread, m = 2, 3:
+// four.  launch_pass_edges: PASS_VEL = their velocities and PASS_STR_LAYER = the
+// stresses that need no velocity of the pass (the radial layer but its rim
+// row), both beside the pass; PASS_STR_RIM = the other stresses, after both.
+inline bool is_pass(int code) { return code > 4000 && code < 4400 && code % 100 >= 1 && code % 100 <= 32; }
+inline int pass_runs(int code) { return code % 100; }
+inline bool pass_per_tile(int code) { return (code / 100) & 1; }
+inline bool pass_edges4(int code) { return code >= 4200; }
+enum { PASS_VEL = 0, PASS_STR_LAYER, PASS_STR_RIM };
+bool pass_region(const KParams &p, int *r1, int *z0, int *z1);
+size_t pass_smem_bytes(int n_mat);  // of one block, the material table included
+// maps: the set read, boxes of 128 z cells x pass_box_rows() rows
+int pass_box_rows();
+cudaError_t launch_pass(int code, const FusedMaps &maps, const PassParams &q, cudaStream_t s);
+cudaError_t launch_pass_edges(int code, int part, const KParams &p, const OutSet &out, cudaStream_t s);
 // single-pass sweep kernel (stencil_sweep.cu): tile code 3000 + 100 m + 10 e
 // + b (b resident blocks per SM, general body in runs of e cells; m: z chunks
 // of 32 or 64 cells, the lag of the stress items, an L2 prefetch of the next

@@ -364,9 +364,12 @@ __device__ __forceinline__ void zero_ids(int (&o)[NV]) {
 // lie inside NZ and outside the z PML (no z memory variable, no z bound
 // check); by default the same as LEAN.  LEAN: the NV cells are interior (no PML
 // memory variable, all inside NZ, k0 + NV < NZ); the kernels pick the lean
-// body per thread, or run it alone on the interior tiles.
+// body per thread, or run it alone on the interior tiles.  out: the set written
+// (null: in place).
 template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN>
-__device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, const int i, const int k0) {
+__device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, const int i, const int k0,
+                                               const OutSet *out = nullptr) {
+  void *const *fo = out ? out->f : p.f;
   const int nth = p.nth, NR = p.NR, NZ = p.NZ;
   const long long NZp = p.NZp, pl = p.plane;
   const int jm = j == 0 ? nth - 1 : j - 1, jp = j == nth - 1 ? 0 : j + 1;
@@ -375,7 +378,7 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
   const long long cjp = (long long)jp * pl + i * NZp + k0;
   const T *srr = (const T *)p.f[F_SRR], *spp = (const T *)p.f[F_SPP], *szz = (const T *)p.f[F_SZZ];
   const T *srp = (const T *)p.f[F_SRP], *spz = (const T *)p.f[F_SPZ], *srz = (const T *)p.f[F_SRZ];
-  T *vr = (T *)p.f[F_VR], *vp = (T *)p.f[F_VP], *vz = (T *)p.f[F_VZ];
+  const T *vr = (const T *)p.f[F_VR], *vp = (const T *)p.f[F_VP], *vz = (const T *)p.f[F_VZ];
   const bool im = i >= 1, ip = i + 1 < NR, k4 = ZIN || k0 + NV < NZ, km = k0 > 0;
 
   // ---- every load
@@ -526,9 +529,10 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
     }
   }
   const SrKey sk = body_key<T>(p, j, i, k0);
-  if (im) st_field<T, NV, false>(vr + c, out_r, sk, F_VR);
-  st_field<T, NV, false>(vp + c, out_p, sk, F_VP);
-  st_field<T, NV, false>(vz + c, out_z, sk, F_VZ);
+  // the axis row's v_r is no unknown: only carried over into another set
+  if (im || out) st_field<T, NV, false>((T *)fo[F_VR] + c, out_r, sk, F_VR);
+  st_field<T, NV, false>((T *)fo[F_VP] + c, out_p, sk, F_VP);
+  st_field<T, NV, false>((T *)fo[F_VZ] + c, out_z, sk, F_VZ);
   if (PRE && rp) {  // cells the loop skipped keep the values loaded
     stv(p.psr[R_VR] + cr, ur_vr);
     stv(p.psr[Q_VR] + cr, uq_vr);
@@ -553,18 +557,21 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
 
 // CG: the velocities are read through L2 only (ldrow / ldone), for a launch
 // in which other blocks wrote them, and the cell's own stresses are read and
-// written streaming (last use in the launch)
+// written streaming (last use in the launch).  out: the set that holds the new
+// velocities and is written (null: in place).
 template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN, bool CG = false>
-__device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, const int i, const int k0) {
+__device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, const int i, const int k0,
+                                               const OutSet *out = nullptr) {
+  void *const *fo = out ? out->f : p.f;
   const int nth = p.nth, NR = p.NR, NZ = p.NZ;
   const long long NZp = p.NZp, pl = p.plane;
   const int jm = j == 0 ? nth - 1 : j - 1, jp = j == nth - 1 ? 0 : j + 1;
   const long long c = (long long)j * pl + i * NZp + k0;
   const long long cjm = (long long)jm * pl + i * NZp + k0;
   const long long cjp = (long long)jp * pl + i * NZp + k0;
-  const T *vr = (const T *)p.f[F_VR], *vp = (const T *)p.f[F_VP], *vz = (const T *)p.f[F_VZ];
-  T *srr = (T *)p.f[F_SRR], *spp = (T *)p.f[F_SPP], *szz = (T *)p.f[F_SZZ];
-  T *srp = (T *)p.f[F_SRP], *spz = (T *)p.f[F_SPZ], *srz = (T *)p.f[F_SRZ];
+  const T *vr = (const T *)fo[F_VR], *vp = (const T *)fo[F_VP], *vz = (const T *)fo[F_VZ];
+  const T *srr = (const T *)p.f[F_SRR], *spp = (const T *)p.f[F_SPP], *szz = (const T *)p.f[F_SZZ];
+  const T *srp = (const T *)p.f[F_SRP], *spz = (const T *)p.f[F_SPZ], *srz = (const T *)p.f[F_SRZ];
   const bool im = i >= 1, ip = i + 1 < NR, k4 = ZIN || k0 + NV < NZ, km = k0 > 0;
 
   // ---- every load
@@ -745,14 +752,14 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
     }
   }
   const SrKey sk = body_key<T>(p, j, i, k0);
-  st_field<T, NV, CG>(srr + c, orr, sk, F_SRR);
-  st_field<T, NV, CG>(spp + c, opp, sk, F_SPP);
-  st_field<T, NV, CG>(szz + c, ozz, sk, F_SZZ);
-  if (im) {
-    st_field<T, NV, CG>(srp + c, orp, sk, F_SRP);
-    st_field<T, NV, CG>(srz + c, orz, sk, F_SRZ);
+  st_field<T, NV, CG>((T *)fo[F_SRR] + c, orr, sk, F_SRR);
+  st_field<T, NV, CG>((T *)fo[F_SPP] + c, opp, sk, F_SPP);
+  st_field<T, NV, CG>((T *)fo[F_SZZ] + c, ozz, sk, F_SZZ);
+  if (im || out) {
+    st_field<T, NV, CG>((T *)fo[F_SRP] + c, orp, sk, F_SRP);
+    st_field<T, NV, CG>((T *)fo[F_SRZ] + c, orz, sk, F_SRZ);
   }
-  st_field<T, NV, CG>(spz + c, opz, sk, F_SPZ);
+  st_field<T, NV, CG>((T *)fo[F_SPZ] + c, opz, sk, F_SPZ);
   if (PRE && rp) {  // cells the loop skipped keep the values loaded
     stv(p.psr[R_ERR] + cr, ur_rr);
     stv(p.psr[Q_EPP] + cr, uq_pp);
@@ -800,7 +807,7 @@ __device__ __forceinline__ void hoist_cells(const KParams &p, int j, int i, int 
 __device__ __forceinline__ void prefetch_l2(const void *a) { asm volatile("prefetch.global.L2 [%0];" ::"l"(a)); }
 
 template <typename T, int NV, bool VEL>
-__device__ __forceinline__ void prefetch_tile(const KParams &p, int j, int i, int k0) {
+__device__ __forceinline__ void prefetch_tile(const KParams &p, int j, int i, int k0, const OutSet *out = nullptr) {
   constexpr int LANES = 128 / (NV * (int)sizeof(T));  // threads per 128-byte line of a field row
   constexpr int LANES_ID = 128 / (NV * 2);
   const long long pl = p.plane, NZp = p.NZp;
@@ -819,10 +826,11 @@ __device__ __forceinline__ void prefetch_tile(const KParams &p, int j, int i, in
       prefetch_l2(f[F_SRP] + cjm), prefetch_l2(f[F_SPZ] + cjm), prefetch_l2(f[F_SPP] + cjp);
     } else {
       for (int q = F_SRR; q <= F_SRZ; q++) prefetch_l2(f[q] + c);
-      prefetch_l2(f[F_VR] + c), prefetch_l2(f[F_VP] + c), prefetch_l2(f[F_VZ] + c);
-      if (ip) prefetch_l2(f[F_VR] + c + NZp);
-      if (im) prefetch_l2(f[F_VP] + c - NZp), prefetch_l2(f[F_VZ] + c - NZp);
-      prefetch_l2(f[F_VP] + cjm), prefetch_l2(f[F_VR] + cjp), prefetch_l2(f[F_VZ] + cjp);
+      const T *const *v = (const T *const *)(out ? out->f : p.f);
+      prefetch_l2(v[F_VR] + c), prefetch_l2(v[F_VP] + c), prefetch_l2(v[F_VZ] + c);
+      if (ip) prefetch_l2(v[F_VR] + c + NZp);
+      if (im) prefetch_l2(v[F_VP] + c - NZp), prefetch_l2(v[F_VZ] + c - NZp);
+      prefetch_l2(v[F_VP] + cjm), prefetch_l2(v[F_VR] + cjp), prefetch_l2(v[F_VZ] + cjp);
     }
   }
   if ((threadIdx.x & (LANES_ID - 1)) == 0) {

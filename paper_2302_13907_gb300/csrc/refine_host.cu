@@ -138,8 +138,8 @@ bool pow2_in(int n) { return n == 4 || n == 8 || n == 16 || n == 32 || n == 64; 
 // zones then run on parallel streams), the fastest pair measured: plain
 // interior + prefetching edge for the velocities, the three-way split for the
 // stresses.  A smaller grid (a 1.6 m crop, several handles side by side) runs
-// all zones of a half in one launch of the batched kernel: 129 us a step of the
-// 136 x 32 x 1330 crop, 178 with two launches per zone and half.
+// all zones of a half in one launch of the batched kernel: 126 us a step of the
+// 136 x 32 x 1330 crop, 176 with two launches per zone and half.
 constexpr int REFINED_VEL_CODE = 2285, REFINED_STR_CODE = 2334;
 constexpr long long ZONE_STREAM_CELLS = 8LL << 20;
 // opts.tile of a refined handle: 0, or a split code or pair code whose halves

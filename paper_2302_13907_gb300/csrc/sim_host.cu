@@ -124,7 +124,7 @@ int cwell::validate_inputs(const sim_grid_t *g, const sim_medium_t *m, const sim
                               (o->kernel == SIM_KERNEL_FUSED_VEC && t >= 100 && t < 1000) ||
                               (o->kernel == SIM_KERNEL_MARCH && is_march(t)) ||
                               (o->kernel == SIM_KERNEL_SWEEP && is_sweep(t)) ||
-                              (o->kernel == SIM_KERNEL_AUTO && (t < 3000 || is_split_pair(t) || is_sweep(t))));
+                              (o->kernel == SIM_KERNEL_AUTO && (t < 3000 || is_split_pair(t) || is_sweep(t) || is_pass(t))));
     if (!ok) return fail(nullptr, SIM_EINVAL, "opts: tile " + std::to_string(t) + " is not a tile code of the kernel asked for");
   }
   if (o->max_steps < 0) return fail(nullptr, SIM_EINVAL, "opts: max_steps < 0");
@@ -254,10 +254,23 @@ static int build_march_maps(sim_t *h, int code) {
   return make_map(h, &h->mmaps.id, h->id, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, march_box_id(), rt + 2);
 }
 
+// descriptors of the one-pass kernel: the stresses of either set (FP32) and the IDs
+static int build_pass_maps(sim_t *h) {
+  for (int par = 0; par < 2; par++) {
+    void **src = par == 0 ? h->f : h->f2;
+    int rc = SIM_OK;
+    for (int q = F_SRR; q < NF && !rc; q++)
+      rc = make_map(h, &h->pmaps[par].f[q], src[q], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, 128, pass_box_rows());
+    if (!rc) rc = make_map(h, &h->pmaps[par].id, h->id, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, 128, pass_box_rows());
+    if (rc) return rc;
+  }
+  return SIM_OK;
+}
+
 // Autotuner: time each tile height on the still-zero state with the source
 // disabled (the state stays zero), keep the fastest; cached per grid shape.
 static std::mutex g_tune_mu;
-static std::map<std::tuple<int, int, int, int, int, int>, int> g_tune;
+static std::map<std::tuple<int, int, int, int, int, int>, std::pair<int, int>> g_tune;  // pick, best split code
 
 static cudaError_t launch_fused_any(int storage, int code, const FusedMaps &maps, const FusedParams &fp,
                                     cudaStream_t s) {
@@ -290,6 +303,56 @@ cudaError_t cwell::sim_split_halves(const sim_t *h, const KParams &p, cudaStream
   return launch_split_family(h->stencil_storage, h->tile_rt, p, s, nullptr, parts);
 }
 
+// One step of the one-pass path from buffer set par to the other: the edge
+// velocities and the radial layer's stresses beside the pass on the side
+// stream (they fill the SMs its last round leaves idle), the stresses that read
+// the pass's velocities after both; a point force on an edge node acts between
+// them, the torsion ring at the end.
+// dry: no source (the tuner's zero state stays zero).
+static cudaError_t launch_pass_step(const sim_t *h, int code, int par, bool dry, cudaEvent_t *ev) {
+  PassParams q = h->pp[par];
+  if (dry) q.k.src_i = q.force_i = -1;
+  const bool outside = h->force_outside && !dry;  // the layer's stresses then wait for the force
+  cudaStream_t s = h->stream;
+  if (ev) cudaEventRecord(ev[0], s);
+  cudaError_t e = cudaEventRecord(h->side.fork, s);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side.side, h->side.fork, 0);
+  if (e == cudaSuccess) e = launch_pass(code, h->pmaps[par], q, s);
+  if (e == cudaSuccess) e = launch_pass_edges(code, PASS_VEL, q.k, q.out, h->side.side);
+  if (e == cudaSuccess && !outside) e = launch_pass_edges(code, PASS_STR_LAYER, q.k, q.out, h->side.side);
+  if (e == cudaSuccess) e = cudaEventRecord(h->side.join, h->side.side);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->side.join, 0);
+  if (e == cudaSuccess && outside) e = launch_inject(h->storage, h->ip2[par], s);
+  if (ev) cudaEventRecord(ev[1], s);
+  if (e == cudaSuccess && outside) e = launch_pass_edges(code, PASS_STR_LAYER, q.k, q.out, s);
+  if (e == cudaSuccess) e = launch_pass_edges(code, PASS_STR_RIM, q.k, q.out, s);
+  if (ev) cudaEventRecord(ev[2], s);
+  if (e == cudaSuccess && !dry && h->src_kind == 3) e = launch_inject(h->storage, h->ip2[par], s);
+  return e;
+}
+
+// time of three replays of four captured steps (each: `step` enqueues step r)
+template <typename F>
+static cudaError_t time_graph(sim_t *h, cudaEvent_t a, cudaEvent_t b, float *ms, F step) {
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
+  for (int r = 0; r < 4 && e == cudaSuccess; r++) e = step(r);
+  cudaError_t e2 = cudaStreamEndCapture(h->stream, &graph);
+  if (e == cudaSuccess) e = e2;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+  if (e == cudaSuccess) e = cudaGraphLaunch(exec, h->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(a, h->stream);
+  for (int r = 0; r < 3 && e == cudaSuccess; r++) e = cudaGraphLaunch(exec, h->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(b, h->stream);
+  if (e == cudaSuccess) e = cudaEventSynchronize(b);
+  if (exec) cudaGraphExecDestroy(exec);
+  if (graph) cudaGraphDestroy(graph);
+  if (e == cudaSuccess) e = cudaEventElapsedTime(ms, a, b);
+  return e;
+}
+
 static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
   SideScope side_scope(h);
   const bool allow_split = kernel == SIM_KERNEL_AUTO || kernel == SIM_KERNEL_SPLIT;
@@ -298,13 +361,14 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
   // point forces rule out the sweep kernel: they key a separate choice
   const bool force = h->src_kind == 1 || h->src_kind == 2;
   auto key = std::make_tuple(dev, h->grid.nth, h->NR, h->NZ, h->stencil_storage * 8 + kernel,
-                             (h->kp.pml_r > 0 ? 1 : 0) + (force ? 2 : 0));
+                             (h->kp.pml_r > 0 ? 1 : 0) + (force ? 2 : 0) + (h->two_sets ? 4 : 0));
   if (!forced) {
     std::lock_guard<std::mutex> g(g_tune_mu);
     auto it = g_tune.find(key);
     if (it != g_tune.end()) {
-      *best_rt = it->second;
-      return SIM_OK;
+      *best_rt = it->second.first;
+      h->split_rt = it->second.second;
+      return is_pass(*best_rt) ? build_pass_maps(h) : SIM_OK;
     }
   }
   const int cand[] = {2,    4,    6,    8,    106,  110,  114,  1216, 1232, 1264, 1416, 1432, 1464, 1816, 1832,
@@ -324,6 +388,15 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
     for (int rt : cand) v |= rt == split_vel_code(forced), c |= rt == split_str_code(forced);
     if (v && c) pick = forced;
   }
+  h->split_rt = 2224;  // half steps beside a forced one-pass code
+  int r1, z0, z1;
+  const bool pass_ok = kernel == SIM_KERNEL_AUTO && h->two_sets && h->storage == SIM_STORAGE_F32 &&
+                       pass_smem_bytes(h->n_mat) <= (size_t)maxsm && pass_region(h->kp, &r1, &z0, &z1);
+  if (pass_ok && (!forced || is_pass(forced))) {
+    int rc = build_pass_maps(h);
+    if (rc) return rc;
+  }
+  if (forced && is_pass(forced) && pass_ok && pass_runs(forced) <= h->grid.nth) pick = forced;
   for (int rt : cand) {
     cudaError_t e = cudaSuccess;
     const bool fused_code = rt < 1000;
@@ -438,38 +511,35 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
       return out;
     };
     const std::vector<int> nv = near(times_v, best_v), ns = near(times_s, best_s);
-    if (nv.size() * ns.size() > 1) {
-      KParams dry = h->kp;
-      dry.src_i = -1;
-      float best_pair = INFINITY;
+    KParams dry = h->kp;
+    dry.src_i = -1;
+    float best_step = INFINITY;
+    cudaError_t e = cudaSuccess;
+    if (pass_ok || nv.size() * ns.size() > 1)
       for (int v : nv)
         for (int c : ns) {
           const int code = v == c ? v : v * 10000 + c;
-          cudaGraph_t graph = nullptr;
-          cudaGraphExec_t exec = nullptr;
-          cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
-          for (int r = 0; r < 4 && e == cudaSuccess; r++)
-            e = launch_split_family(h->stencil_storage, code, dry, h->stream, nullptr);
-          cudaError_t e2 = cudaStreamEndCapture(h->stream, &graph);
-          if (e == cudaSuccess) e = e2;
-          if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-          if (e == cudaSuccess) e = cudaGraphLaunch(exec, h->stream);
-          if (e == cudaSuccess) e = cudaEventRecord(a, h->stream);
-          for (int r = 0; r < 3 && e == cudaSuccess; r++) e = cudaGraphLaunch(exec, h->stream);
-          if (e == cudaSuccess) e = cudaEventRecord(b, h->stream);
-          if (e == cudaSuccess) e = cudaEventSynchronize(b);
-          if (exec) cudaGraphExecDestroy(exec);
-          if (graph) cudaGraphDestroy(graph);
-          if (e != cudaSuccess) {
-            cudaEventDestroy(a);
-            cudaEventDestroy(b);
-            cudaEventDestroy(c3);
-            return cuda_fail(h, e, "autotune graph");
-          }
           float ms = 0;
-          cudaEventElapsedTime(&ms, a, b);
-          if (ms < best_pair) best_pair = ms, pick = code;
+          if (e == cudaSuccess)
+            e = time_graph(h, a, b, &ms, [&](int) { return launch_split_family(h->stencil_storage, code, dry, h->stream, nullptr); });
+          if (e == cudaSuccess && ms < best_step) best_step = ms, pick = code;
         }
+    h->split_rt = pick;
+    // the one-pass step against the best pair: ahead from some 3 M cells on (88 x 22
+    // x 1527 cells 75 us a step against 79), behind where a march is short and the
+    // state stays in L2 anyway (70 x 16 x 320 cells 18.8 us against 14.6)
+    if (pass_ok)
+      for (int code : {4001, 4101, 4201, 4301}) {
+        float ms = 0;
+        if (2 * pass_runs(code) > h->grid.nth || e != cudaSuccess) continue;
+        e = time_graph(h, a, b, &ms, [&](int r) { return launch_pass_step(h, code, r & 1, true, nullptr); });
+        if (e == cudaSuccess && ms < best_step) best_step = ms, pick = code;
+      }
+    if (e != cudaSuccess) {
+      cudaEventDestroy(a);
+      cudaEventDestroy(b);
+      cudaEventDestroy(c3);
+      return cuda_fail(h, e, "autotune graph");
     }
   }
   cudaEventDestroy(a);
@@ -480,7 +550,7 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
   if (pick < 0) return fail(h, SIM_EUNSUPPORTED, "no tile of the requested kernel fits in shared memory");
   if (!forced) {
     std::lock_guard<std::mutex> g(g_tune_mu);
-    g_tune[key] = pick;
+    g_tune[key] = {pick, h->split_rt};
   }
   *best_rt = pick;
   return SIM_OK;
@@ -736,6 +806,20 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
         if ((rc = dev_alloc(h, (void **)&h->psz2[q], h->psz_elems * 4))) return bail(rc);
     }
   }
+  h->two_sets = h->fused;
+  if (opts->kernel == SIM_KERNEL_AUTO && !h->fused && !slab && opts->storage == SIM_STORAGE_F32 && source->kind != 0) {
+    // the point forces and the torsion ring rule out the fused kernels but not
+    // the one-pass step: it gets its second set where that takes no more than a
+    // third of the free memory and stays under the cap
+    const size_t set = NF * ((fbytes + 255) & ~size_t(255));
+    size_t free_b = 0, total_b = 0;
+    if ((e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bail(cuda_fail(h, e, "cudaMemGetInfo"));
+    if (3 * set <= free_b && (!h->mem_cap || h->bytes + 2 * set <= h->mem_cap)) {
+      for (int q = 0; q < NF; q++)
+        if ((rc = dev_alloc(h, &h->f2[q], fbytes))) return bail(rc);
+      h->two_sets = true;
+    }
+  }
   if ((rc = dev_alloc(h, (void **)&h->id, (size_t)nth * NR * NZp * 2))) return bail(rc);
   if ((rc = dev_alloc(h, (void **)&h->mat, mat.size() * sizeof(float4)))) return bail(rc);
   if ((rc = dev_alloc(h, (void **)&h->m_rho, mat.size() * 4))) return bail(rc);
@@ -837,6 +921,21 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
   h->ip.n_wav = h->n_wav;
   h->ip.step = h->step;
   for (int q = 0; q < NF; q++) h->ip.f[q] = h->f[q];
+  std::vector<float> fw;  // point force: weight of each azimuthal node
+  float *d_fw = nullptr;
+  int force_i = -1;
+  if ((source->kind == 1 || source->kind == 2) && !ifld.empty() && h->two_sets) {
+    fw.assign(nth, 0.f);
+    for (size_t q = 0; q < ioff.size(); q++) {
+      const int j = (int)(ioff[q] / p.plane);
+      force_i = (int)(ioff[q] % p.plane / NZp);
+      fw[j] = iw[q];
+    }
+    if ((rc = dev_alloc(h, (void **)&d_fw, nth * 4))) return bail(rc);
+    if ((e = cudaMemcpyAsync(d_fw, fw.data(), nth * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(st)) != cudaSuccess)
+      return bail(cuda_fail(h, e, "upload force"));
+  }
   RParams &r = h->rp;
   r.nth = nth;
   r.NR = NR;
@@ -852,6 +951,30 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
   r.traces = h->traces;
   r.step = h->step;
   r.status = h->status;
+  if (h->two_sets)
+    for (int par = 0; par < 2; par++) {  // step from set par to the other
+      PassParams &q = h->pp[par];
+      void **cur = par == 0 ? h->f : h->f2, **nxt = par == 0 ? h->f2 : h->f;
+      q.k = p;
+      h->ip2[par] = h->ip;
+      for (int k = 0; k < NF; k++) {
+        q.k.f[k] = cur[k];
+        q.out.f[k] = h->ip2[par].f[k] = nxt[k];
+      }
+      q.status = h->status;
+      q.n_mat = h->n_mat;
+      q.force_i = force_i;
+      q.force_k = (int)ks - l0;
+      q.force_vz = source->kind == 2;
+      q.force_w = d_fw;
+      q.force_wav = d_iwav;
+      h->rp2[par] = r;
+      h->rp2[par].srr = nxt[F_SRR];
+      h->rp2[par].spp = nxt[F_SPP];
+      h->rp2[par].szz = nxt[F_SZZ];
+      int r1, z0, z1;
+      h->force_outside = force_i >= 0 && !(pass_region(q.k, &r1, &z0, &z1) && force_i < r1 && q.force_k >= z0 && q.force_k < z1);
+    }
   if (opts->watchdog_every > 0) {
     h->watch_every = opts->watchdog_every;
     if ((rc = dev_alloc(h, (void **)&h->watch_acc, 4 * sizeof(double)))) return bail(rc);
@@ -870,9 +993,7 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
       w.every = h->watch_every;
       // the last step of the source's wavelet tables: no injection after it
       w.n_quiet = std::max(h->n_wav, h->ip.n_wav);
-      // the state after a step of parity par (the fused path writes the other set)
-      void **cur = (h->fused && par == 0) ? h->f2 : h->f;
-      for (int q = 0; q < NF; q++) w.f[q] = cur[q];
+      for (int q = 0; q < NF; q++) w.f[q] = h->f[q];  // in place; the paths with two sets below
       w.id = h->id;
       w.m_rho = h->m_rho;
       w.m_lam = h->m_lam;
@@ -903,16 +1024,14 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
         f.psz_o[q] = zn[q];
       }
       f.status = h->status;
-      // the stresses of step n + 1 are in the buffer this parity writes
-      h->rp2[par] = r;
-      h->rp2[par].srr = nxt[F_SRR];
-      h->rp2[par].spp = nxt[F_SPP];
-      h->rp2[par].szz = nxt[F_SZZ];
     }
     if ((rc = autotune(h, opts->kernel, opts->tile, &h->tile_rt))) return bail(rc);
     if (is_split_family(h->tile_rt)) {  // the split kernels won: run in place on the first buffer set
       h->fused = false;
       h->kernel = SIM_KERNEL_SPLIT;
+    } else if (is_pass(h->tile_rt)) {  // the one-pass step won
+      h->fused = false;
+      h->pass = true;
     } else if (is_sweep(h->tile_rt)) {  // the sweep kernel won: in place as well
       h->fused = false;
       h->kernel = SIM_KERNEL_SWEEP;
@@ -928,9 +1047,14 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
     if ((rc = autotune(h, h->kernel, opts->tile, &h->tile_rt))) return bail(rc);
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return bail(cuda_fail(h, e, "autotune"));
+    h->pass = is_pass(h->tile_rt);
     h->kernel = is_march(h->tile_rt) ? SIM_KERNEL_MARCH : is_sweep(h->tile_rt) ? SIM_KERNEL_SWEEP : SIM_KERNEL_SPLIT;
   }
   h->sweep = h->kernel == SIM_KERNEL_SWEEP;
+  if (h->pass) h->kernel = SIM_KERNEL_ONEPASS;
+  if (h->fused || h->pass)  // the watchdog sees the set a step of parity par writes
+    for (int par = 0; par < 2; par++)
+      for (int q = 0; q < NF; q++) h->wp[par].f[q] = par == 0 ? h->f2[q] : h->f[q];
   if (h->kernel == SIM_KERNEL_MARCH) {
     h->march = true;
     if ((rc = build_march_maps(h, h->tile_rt))) return bail(rc);
@@ -967,6 +1091,9 @@ static cudaError_t enqueue_step(sim_t *h, int parity, bool timed) {
       cudaEventRecord(h->ev[2], h->stream);
     }
     e = launch_receivers(h->storage, h->rp2[parity], h->stream);
+  } else if (h->pass) {
+    e = launch_pass_step(h, h->tile_rt, parity, false, timed ? h->ev : nullptr);
+    if (e == cudaSuccess) e = launch_receivers(h->storage, h->rp2[parity], h->stream);
   } else if (h->sweep) {
     if (timed) cudaEventRecord(h->ev[0], h->stream);
     e = launch_sweep(h->stencil_storage, h->tile_rt, h->kp, h->vdone, h->status, h->wait_cycles, h->withhold_chunk,
@@ -1025,18 +1152,22 @@ extern "C" int sim_step(sim_t *h, int nsteps) {
   if (nsteps < 0) return fail(h, SIM_EINVAL, "nsteps < 0");
   CK(h, cudaSetDevice(h->device));
   int left = nsteps;
+  // the set a step starts from: the fused kernels alternate with the step
+  // number, the one-pass path with its own steps (half steps stay in place)
+  auto parity = [&] { return h->pass ? h->cur : h->steps_done & 1; };
   auto direct = [&]() -> int {
-    cudaError_t e = enqueue_step(h, h->steps_done & 1, h->timing != 0);
+    cudaError_t e = enqueue_step(h, parity(), h->timing != 0);
     if (e != cudaSuccess) return cuda_fail(h, e, "kernel launch");
+    if (h->pass) h->cur ^= 1;
     h->steps_done++;
     left--;
     return SIM_OK;
   };
   // a captured chunk starts on an even step (fused buffers alternate) and has even length
   int chunk = h->graph_chunk;
-  if (h->fused && chunk > 0 && (chunk & 1)) chunk++;
-  if (!h->timing && chunk > 0 && left >= chunk + (h->steps_done & 1)) {
-    if (h->steps_done & 1) {
+  if ((h->fused || h->pass) && chunk > 0 && (chunk & 1)) chunk++;
+  if (!h->timing && chunk > 0 && left >= chunk + parity()) {
+    if (parity()) {
       int rc = direct();
       if (rc) return rc;
     }
@@ -1066,8 +1197,9 @@ extern "C" int sim_step(sim_t *h, int nsteps) {
   return SIM_OK;
 }
 
-// buffers holding the current state (the fused path alternates two sets)
-static void **cur_fields(sim_t *h) { return (h->fused && (h->steps_done & 1)) ? h->f2 : h->f; }
+// buffers holding the current state (the fused path alternates two sets of
+// everything, the one-pass path two sets of the fields)
+static void **cur_fields(sim_t *h) { return (h->fused && (h->steps_done & 1)) || (h->pass && h->cur) ? h->f2 : h->f; }
 static float **cur_psr(sim_t *h) { return (h->fused && (h->steps_done & 1)) ? h->psr2 : h->psr; }
 static float **cur_psz(sim_t *h) { return (h->fused && (h->steps_done & 1)) ? h->psz2 : h->psz; }
 
@@ -1078,10 +1210,17 @@ extern "C" int sim_half_step(sim_t *h, int which) {
   CK(h, cudaSetDevice(h->device));
   SideScope side_scope(h);
   const bool force = h->src_kind == 1 || h->src_kind == 2;
-  cudaError_t e = launch_split_family(h->stencil_storage, h->tile_rt, h->kp, h->stream, nullptr, which == 0 ? 1 : 2);
-  if (e == cudaSuccess && ((which == 0 && force) || (which == 1 && h->src_kind == 3)))
-    e = launch_inject(h->storage, h->ip, h->stream);
-  if (e == cudaSuccess && which == 1) e = launch_receivers(h->storage, h->rp, h->stream);
+  KParams kp = h->kp;
+  IParams ip = h->ip;
+  RParams rp = h->rp;
+  if (h->pass && h->cur) {  // in place on the set that holds the state
+    for (int q = 0; q < NF; q++) kp.f[q] = ip.f[q] = h->f2[q];
+    rp = h->rp2[0];
+  }
+  cudaError_t e = launch_split_family(h->stencil_storage, h->pass ? h->split_rt : h->tile_rt, kp, h->stream, nullptr,
+                                      which == 0 ? 1 : 2);
+  if (e == cudaSuccess && ((which == 0 && force) || (which == 1 && h->src_kind == 3))) e = launch_inject(h->storage, ip, h->stream);
+  if (e == cudaSuccess && which == 1) e = launch_receivers(h->storage, rp, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "half step");
   if (which == 1) h->steps_done++;
   return SIM_OK;
@@ -1108,7 +1247,7 @@ static int copy_planes(sim_t *h, int group, int k0, int k1, void *buf, bool out)
   const int q0 = group == 0 ? F_VR : F_SRR, q1 = group == 0 ? F_SRR : NF;
   const size_t w = (size_t)(k1 - k0) * h->elem, rows = (size_t)h->grid.nth * h->NR;
   for (int q = q0; q < q1; q++) {
-    char *f = (char *)h->f[q] + (size_t)(k0 - h->l0) * h->elem;
+    char *f = (char *)cur_fields(h)[q] + (size_t)(k0 - h->l0) * h->elem;
     char *b = (char *)buf + (size_t)(q - q0) * rows * w;
     cudaError_t e = out ? cudaMemcpy2DAsync(b, w, f, (size_t)h->NZp * h->elem, w, rows, cudaMemcpyDefault, h->stream)
                         : cudaMemcpy2DAsync(f, (size_t)h->NZp * h->elem, b, w, w, rows, cudaMemcpyDefault, h->stream);

@@ -57,6 +57,15 @@ struct sim_s {
   bool march = false;
   FusedMaps mmaps;
   FusedParams fp[2];
+  // one-pass path: the state alternates between the two field sets (memory
+  // variables in place); cur = the set that holds it.  two_sets: the second
+  // set exists; split_rt: the split code of sim_half_step
+  bool pass = false, two_sets = false;
+  int cur = 0, split_rt = 0;
+  PassParams pp[2]{};
+  FusedMaps pmaps[2];
+  IParams ip2[2]{};
+  bool force_outside = false;  // the point force's node lies outside the pass region
   RParams rp2[2];
   // second stream and fork / join events of the three-way split halves
   SideStream side{};

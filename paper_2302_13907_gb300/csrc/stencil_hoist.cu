@@ -61,22 +61,22 @@ __global__ void __launch_bounds__(HB_X *HB_Y, MINB) str_hoist(const KParams p) {
 // general body instead of pml_z: 16 % of a 1527-cell row, all of a 256-cell
 // one.)
 struct Regions {
+  int r0;            // first row of the radial layer
   int za, zb;        // lean z groups
   int zt0, nzt, nrt; // interior tiles: z tiles zt0 .. zt0 + nzt - 1, r tiles 0 .. nrt - 1 from row i_lo
-  int rzt0, rnzt, rnrt;  // radial tiles: the same, r tiles counted from row nr
+  int rzt0, rnzt, rnrt;  // radial tiles: the same, r tiles counted from row r0
   int na, nb;        // groups per row of the low and the high z end
   long long interior, radial, ends;  // tiles, tiles, blocks of 128 threads
 };
 
-// NV: cells per thread in the interior, NVE: in the radial layer and the z ends
+// tiles of the regions r0, za, zb; NV: cells per thread in the interior, NVE:
+// in the radial layer and the z ends
 template <int NV, int NVE>
-__host__ Regions regions(const KParams &p) {
+Regions region_tiles(const KParams &p, int r0, int za, int zb) {
   Regions q;
-  q.za = (p.pml_z + 3) / 4 * 4;
-  q.zb = std::max(q.za, (p.NZ - p.pml_z - 1) / 4 * 4);
-  constexpr int W = NV * HB_X;
-  if (q.za % W > W - W / 4) q.za = (q.za + W - 1) / W * W;
-  if (q.zb % W < W / 4) q.zb = std::max(q.za, q.zb / W * W);
+  q.r0 = r0;
+  q.za = za;
+  q.zb = zb;
   const bool any = q.zb > q.za;
   auto tiles = [&](int w, int &t0, int &n) {
     t0 = q.za / w;
@@ -84,14 +84,23 @@ __host__ Regions regions(const KParams &p) {
   };
   tiles(NV * HB_X, q.zt0, q.nzt);
   tiles(NVE * HB_X, q.rzt0, q.rnzt);
-  q.nrt = (std::max(0, std::min(std::min(p.nr, p.NR), p.i_hi) - p.i_lo) + HB_Y - 1) / HB_Y;
-  q.rnrt = p.NR > p.nr ? (p.NR - p.nr + HB_Y - 1) / HB_Y : 0;
+  q.nrt = (std::max(0, std::min(r0, p.i_hi) - p.i_lo) + HB_Y - 1) / HB_Y;
+  q.rnrt = (p.NR - r0 + HB_Y - 1) / HB_Y;
   q.na = q.za / NVE;
   q.nb = (p.NZ - q.zb + NVE - 1) / NVE;
   q.interior = (long long)p.nth * q.nrt * q.nzt;
   q.radial = (long long)p.nth * q.rnrt * q.rnzt;
   q.ends = ((long long)p.nth * (p.i_hi - p.i_lo) * (q.na + q.nb) + HB_X * HB_Y - 1) / (HB_X * HB_Y);
   return q;
+}
+
+template <int NV, int NVE>
+Regions regions(const KParams &p) {
+  int za = (p.pml_z + 3) / 4 * 4, zb = std::max(za, (p.NZ - p.pml_z - 1) / 4 * 4);
+  constexpr int W = NV * HB_X;
+  if (za % W > W - W / 4) za = (za + W - 1) / W * W;
+  if (zb % W < W / 4) zb = zb / W * W;
+  return region_tiles<NV, NVE>(p, std::min(p.nr, p.NR), za, std::max(za, zb));
 }
 
 // cell group of this thread in interior tile t (theta fastest, then r, then z); false: nothing to do
@@ -101,13 +110,13 @@ __device__ __forceinline__ bool interior_cell(const KParams &p, const Regions &q
   t /= p.nth;
   i = p.i_lo + (t % q.nrt) * HB_Y + threadIdx.y;
   k0 = ((q.zt0 + t / q.nrt) * HB_X + threadIdx.x) * NV;
-  return i < p.nr && i < p.i_hi && k0 >= q.za && k0 < q.zb && k0 >= p.k_lo && k0 < p.k_hi;
+  return i < q.r0 && i < p.i_hi && k0 >= q.za && k0 < q.zb && k0 >= p.k_lo && k0 < p.k_hi;
 }
 template <int NV>
 __device__ __forceinline__ bool radial_cell(const KParams &p, const Regions &q, int t, int &j, int &i, int &k0) {
   j = t % p.nth;
   t /= p.nth;
-  i = p.nr + (t % q.rnrt) * HB_Y + threadIdx.y;
+  i = q.r0 + (t % q.rnrt) * HB_Y + threadIdx.y;
   k0 = ((q.rzt0 + t / q.rnrt) * HB_X + threadIdx.x) * NV;
   return i >= p.i_lo && i < p.i_hi && k0 >= q.za && k0 < q.zb && k0 >= p.k_lo && k0 < p.k_hi;
 }
@@ -129,14 +138,14 @@ __device__ __forceinline__ void lean_cells_step(const KParams &p, int j, int i, 
   else str_hoist_body<T, NV, true>(p, j, i, k0);
 }
 template <typename T, int NV, bool VEL>
-__device__ __forceinline__ void radial_cells_step(const KParams &p, int j, int i, int k0) {
-  if (VEL) vel_hoist_body<T, NV, false, true, true>(p, j, i, k0);
-  else str_hoist_body<T, NV, false, true, true>(p, j, i, k0);
+__device__ __forceinline__ void radial_cells_step(const KParams &p, int j, int i, int k0, const OutSet *out = nullptr) {
+  if (VEL) vel_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
+  else str_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
 }
 template <typename T, int NV, bool VEL>
-__device__ __forceinline__ void end_cells_step(const KParams &p, int j, int i, int k0) {
-  if (VEL) vel_hoist_body<T, NV, false, true>(p, j, i, k0);
-  else str_hoist_body<T, NV, false, true>(p, j, i, k0);
+__device__ __forceinline__ void end_cells_step(const KParams &p, int j, int i, int k0, const OutSet *out = nullptr) {
+  if (VEL) vel_hoist_body<T, NV, false, true>(p, j, i, k0, out);
+  else str_hoist_body<T, NV, false, true>(p, j, i, k0, out);
 }
 
 template <typename T, int NV, int MINB, bool VEL>
@@ -162,10 +171,10 @@ __global__ void __launch_bounds__(HB_X *HB_Y, MINB) hoist_interior_pf(const KPar
 
 // L2 prefetch of a radial-layer tile: the fields' rows and the memory variables
 template <typename T, int NV, bool VEL>
-__device__ __forceinline__ void prefetch_radial(const KParams &p, int j, int i, int k0) {
+__device__ __forceinline__ void prefetch_radial(const KParams &p, int j, int i, int k0, const OutSet *out = nullptr) {
   constexpr int LANES = 128 / (NV * 4);
-  prefetch_tile<T, NV, VEL>(p, j, i, k0);
-  if ((threadIdx.x & (LANES - 1)) == 0) {
+  prefetch_tile<T, NV, VEL>(p, j, i, k0, out);
+  if (i >= p.nr && (threadIdx.x & (LANES - 1)) == 0) {
     const long long cr = ((long long)j * p.pml_r + (i - p.nr)) * p.NZp + k0;
     const int q0 = VEL ? R_VR : R_ERR, q1 = VEL ? Q_VR : Q_EPP;
     for (int u = 0; u < 3; u++) prefetch_l2(p.psr[q0 + u] + cr), prefetch_l2(p.psr[q1 + u] + cr);
@@ -190,19 +199,35 @@ __global__ void __launch_bounds__(HB_X *HB_Y, MINB) hoist_ends(const KParams p, 
 }
 
 // z ends (first blocks) and radial layer in one launch; PF: the radial tiles
-// are walked by the blocks left in one wave, prefetching the next tile
-template <typename T, int NV, int MINB, bool VEL, bool PF>
-__global__ void __launch_bounds__(HB_X *HB_Y, MINB) hoist_edge(const KParams p, const Regions q) {
+// are walked by the blocks left in one wave, prefetching the next tile; OUT:
+// out of place into `out`
+template <typename T, int NV, int MINB, bool VEL, bool PF, bool OUT = false>
+__global__ void __launch_bounds__(HB_X *HB_Y, MINB) hoist_edge(const KParams p, const Regions q, const OutSet set) {
+  const OutSet *out = OUT ? &set : nullptr;
   int j, i, k0;
   if (blockIdx.x < q.ends) {
-    if (end_cell<NV>(p, q, blockIdx.x, j, i, k0)) end_cells_step<T, NV, VEL>(p, j, i, k0);
+    if (end_cell<NV>(p, q, blockIdx.x, j, i, k0)) end_cells_step<T, NV, VEL>(p, j, i, k0, out);
     return;
   }
   const int n = (int)q.radial, step = gridDim.x - (int)q.ends;
   for (int t = blockIdx.x - (int)q.ends; t < n; t += step) {
-    if (PF && t + step < n && radial_cell<NV>(p, q, t + step, j, i, k0)) prefetch_radial<T, NV, VEL>(p, j, i, k0);
-    if (radial_cell<NV>(p, q, t, j, i, k0)) radial_cells_step<T, NV, VEL>(p, j, i, k0);
+    if (PF && t + step < n && radial_cell<NV>(p, q, t + step, j, i, k0)) prefetch_radial<T, NV, VEL>(p, j, i, k0, out);
+    if (radial_cell<NV>(p, q, t, j, i, k0)) radial_cells_step<T, NV, VEL>(p, j, i, k0, out);
   }
+}
+
+// z ends (first blocks) and the row q.r0 alone, four z tiles per block, out of place
+template <typename T, int NV, int MINB, bool VEL>
+__global__ void __launch_bounds__(HB_X *HB_Y, MINB) hoist_rim(const KParams p, const Regions q, const OutSet set) {
+  int j, i, k0;
+  if (blockIdx.x < q.ends) {
+    if (end_cell<NV>(p, q, blockIdx.x, j, i, k0)) end_cells_step<T, NV, VEL>(p, j, i, k0, &set);
+    return;
+  }
+  const int t = blockIdx.x - (int)q.ends;
+  j = t % p.nth;
+  k0 = ((q.rzt0 + t / p.nth * HB_Y + threadIdx.y) * HB_X + threadIdx.x) * NV;
+  if (k0 >= q.za && k0 < q.zb) radial_cells_step<T, NV, VEL>(p, j, q.r0, k0, &set);
 }
 
 // the whole half step in one launch: z ends, radial layer, interior, in this
@@ -350,7 +375,7 @@ cudaError_t launch_split_half(const KParams &p, const Regions &q, cudaStream_t s
   if (e != cudaSuccess) return e;
   if constexpr (MINB_R == 0) {
     const int rad = PFE ? wave(q.radial, MINB_E) : (int)q.radial;
-    if (edge) hoist_edge<T, NVE, MINB_E, VEL, PFE><<<(int)q.ends + rad, blk, 0, se>>>(p, q);
+    if (edge) hoist_edge<T, NVE, MINB_E, VEL, PFE><<<(int)q.ends + rad, blk, 0, se>>>(p, q, OutSet{});
   } else {
     if (q.radial > 0) hoist_radial_pf<T, NVE, MINB_R, VEL><<<wave(q.radial, MINB_R), blk, 0, se>>>(p, q);
     if (q.ends > 0) hoist_ends<T, NVE, MINB_E, VEL><<<(int)q.ends, blk, 0, se>>>(p, q);
@@ -413,6 +438,27 @@ cudaError_t launch_hoist_t(const KParams &p, cudaStream_t s, cudaEvent_t *ev, in
     str_hoist<T, NV, MINB, ZF><<<grd, blk, 0, s>>>(p);
     if (ev) cudaEventRecord(ev[2], s);
   }
+  return cudaGetLastError();
+}
+
+// the cells beside a one-pass step's: z ends, radial layer and its rim row r1
+template <int NV, int MINB>
+cudaError_t launch_pass_edges_t(int part, const KParams &p, const OutSet &out, cudaStream_t s) {
+  int r1, z0, z1;
+  if (!pass_region(p, &r1, &z0, &z1)) return cudaErrorInvalidValue;
+  const dim3 blk(HB_X, HB_Y);
+  Regions q = region_tiles<4, NV>(p, part == PASS_STR_LAYER ? std::min(r1 + 1, p.NR) : r1, z0, z1);
+  if (!fits(q)) return cudaErrorInvalidValue;
+  if (part == PASS_STR_RIM) {
+    const long long rim = r1 < p.NR ? (long long)p.nth * ((q.rnzt + HB_Y - 1) / HB_Y) : 0;
+    if (q.ends + rim > 0) hoist_rim<float, NV, MINB, false><<<(int)(q.ends + rim), blk, 0, s>>>(p, q, out);
+    return cudaGetLastError();
+  }
+  if (part == PASS_STR_LAYER) q.ends = 0;
+  const int grid = (int)q.ends + wave(q.radial, MINB);
+  if (grid == 0) return cudaSuccess;
+  if (part == PASS_VEL) hoist_edge<float, NV, MINB, true, true, true><<<grid, blk, 0, s>>>(p, q, out);
+  else hoist_edge<float, NV, MINB, false, true, true><<<grid, blk, 0, s>>>(p, q, out);
   return cudaGetLastError();
 }
 
@@ -502,6 +548,10 @@ cudaError_t launch_sr_round(const float *x, const unsigned *dither, unsigned sho
   const int grid = (int)std::min<long long>((n + 255) / 256, 152LL * 8);
   sr_round_kernel<<<grid, 256, 0, s>>>(x, dither, out, n);
   return cudaGetLastError();
+}
+
+cudaError_t launch_pass_edges(int code, int part, const KParams &p, const OutSet &out, cudaStream_t s) {
+  return pass_edges4(code) ? launch_pass_edges_t<4, 3>(part, p, out, s) : launch_pass_edges_t<2, 4>(part, p, out, s);
 }
 
 cudaError_t launch_hoist(int storage, int code, const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts) {
