@@ -185,12 +185,20 @@ __device__ __forceinline__ void ld_ids(const uint16_t *p, int (&o)[4]) {
   o[3] = u.y >> 16;
 }
 
+// 1 / x by the reciprocal unit (1 ulp; +inf gives 0), without the scaling of
+// large and tiny divisors that the division intrinsic adds: none of the sums
+// below is near either
+__device__ __forceinline__ float rcp_fast(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 // velocity coefficient 2 dt / (rho_a + rho_b) (two-cell mean density) and
-// four-cell harmonic shear modulus 4 / sum(1/mu), by the fast division
-// intrinsic (within 2 ulp; the coefficients need no more).  A liquid among the
-// four cells makes the sum +inf and the modulus exactly 0.
-__device__ __forceinline__ float vel_coef(float dtv, float rho_sum) { return __fdividef(2.f * dtv, rho_sum); }
-__device__ __forceinline__ float mu_harm(float imu_sum) { return __fdividef(4.f, imu_sum); }
+// four-cell harmonic shear modulus 4 / sum(1/mu) (within 2 ulp; the
+// coefficients need no more).  A liquid among the four cells makes the sum
+// +inf and the modulus exactly 0.
+__device__ __forceinline__ float vel_coef(float dtv, float rho_sum) { return 2.f * dtv * rcp_fast(rho_sum); }
+__device__ __forceinline__ float mu_harm(float imu_sum) { return 4.f * rcp_fast(imu_sum); }
 
 // convolutional memory variable: psi <- b psi + a D, returns D + psi
 __device__ __forceinline__ float stretch(float *psi, float a, float b, float D) {

@@ -113,12 +113,6 @@ __device__ __forceinline__ PassItem pass_item(const PassParams &q, int R, int t)
   return it;
 }
 
-// 1 / x, 1 ulp; +inf gives 0 (a liquid among the cells of a shear modulus)
-__device__ __forceinline__ float rcp_fast(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 // an old velocity: used once, kept out of the way in L1
 __device__ __forceinline__ void ld_once(float (&d)[4], const float *p) {
   asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
