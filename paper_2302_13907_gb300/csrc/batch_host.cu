@@ -26,6 +26,9 @@ struct simb_s {
   static constexpr int MAX_BRANCH = 4;
   cudaStream_t branch[MAX_BRANCH] = {};
   cudaEvent_t fork = nullptr, join[MAX_BRANCH] = {};
+  // captured chunks: the receivers of a step run beside the next one's first half
+  SideStream rec_side{};
+  bool rec_pending = false;
   int nbranch = 1;
   bool fixed_branches = false;
   cudaGraphExec_t gexec = nullptr;
@@ -53,6 +56,9 @@ static void brelease(simb_t *b) {
     if (b->join[k]) cudaEventDestroy(b->join[k]);
   }
   if (b->fork) cudaEventDestroy(b->fork);
+  if (b->rec_side.fork) cudaEventDestroy(b->rec_side.fork);
+  if (b->rec_side.join) cudaEventDestroy(b->rec_side.join);
+  if (b->rec_side.side) cudaStreamDestroy(b->rec_side.side);
   for (sim_t *h : b->cases) sim_destroy(h);
   b->cases.clear();
   if (b->d_rp) cudaFree(b->d_rp);
@@ -79,6 +85,11 @@ static cudaError_t batch_step(simb_t *b, const KParams *cases) {
     for (int k = 0; k < nb && e == cudaSuccess; k++) e = cudaStreamWaitEvent(b->branch[k], b->fork, 0);
   }
   for (int half = 1; half <= 2 && e == cudaSuccess; half++) {
+    if (half == 2 && b->rec_pending) {  // the samples of the step before are taken from these stresses
+      e = cudaStreamWaitEvent(b->stream, b->rec_side.join, 0);
+      for (int k = 0; k < nb && nb > 1 && e == cudaSuccess; k++) e = cudaStreamWaitEvent(b->branch[k], b->rec_side.join, 0);
+      if (e != cudaSuccess) break;
+    }
     if (!sh.empty()) e = launch_batch_split(b->storage, half == 1, sh.data(), (int)sh.size(), b->stream);
     for (size_t q = 0; q < b->own.size() && e == cudaSuccess; q++)
       e = sim_split_halves(b->cases[b->own[q]], cases[b->own[q]], stream_of(q), half);
@@ -168,7 +179,10 @@ extern "C" int simb_create(int n, const sim_grid_t *grids, const sim_medium_t *m
     if (e != cudaSuccess) return bail(bcuda(b, e, "cudaStreamCreate"));
     b->own_stream = true;
   }
-  if ((e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming)) != cudaSuccess)
+  if ((e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming)) != cudaSuccess ||
+      (e = cudaEventCreateWithFlags(&b->rec_side.fork, cudaEventDisableTiming)) != cudaSuccess ||
+      (e = cudaEventCreateWithFlags(&b->rec_side.join, cudaEventDisableTiming)) != cudaSuccess ||
+      (e = cudaStreamCreateWithFlags(&b->rec_side.side, cudaStreamNonBlocking)) != cudaSuccess)
     return bail(bcuda(b, e, "cudaEventCreate"));
   for (int k = 0; k < simb_t::MAX_BRANCH; k++)
     if ((e = cudaStreamCreateWithFlags(&b->branch[k], cudaStreamNonBlocking)) != cudaSuccess ||
@@ -223,10 +237,20 @@ extern "C" int simb_create(int n, const sim_grid_t *grids, const sim_medium_t *m
   return SIM_OK;
 }
 
-static cudaError_t enqueue_batch_step(simb_t *b) {
-  cudaError_t e = batch_step(b, b->kp.data());
-  if (e == cudaSuccess) e = launch_batch_receivers(b->storage, b->d_rp, (int)b->cases.size(), b->stream);
-  return e;
+// off >= 0: step `off` of a captured chunk, the receivers beside the next step's
+// velocity half (see enqueue_step of the single well); off < 0: a step by itself
+static cudaError_t enqueue_batch_step(simb_t *b, int off) {
+  std::vector<KParams> kp = b->kp;
+  for (KParams &p : kp) p.step_off = std::max(off, 0);
+  const int n = (int)b->cases.size();
+  cudaError_t e = batch_step(b, kp.data());
+  if (e != cudaSuccess || off < 0)
+    return e != cudaSuccess ? e : launch_batch_receivers(b->storage, b->d_rp, n, 0, true, b->stream);
+  if ((e = cudaEventRecord(b->rec_side.fork, b->stream)) != cudaSuccess) return e;
+  if ((e = cudaStreamWaitEvent(b->rec_side.side, b->rec_side.fork, 0)) != cudaSuccess) return e;
+  if ((e = launch_batch_receivers(b->storage, b->d_rp, n, off, false, b->rec_side.side)) != cudaSuccess) return e;
+  b->rec_pending = true;
+  return cudaEventRecord(b->rec_side.join, b->rec_side.side);
 }
 
 extern "C" int simb_run(simb_t *b, int nsteps) {
@@ -241,7 +265,10 @@ extern "C" int simb_run(simb_t *b, int nsteps) {
       if ((e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
         return bcuda(b, e, "cudaStreamBeginCapture");
       cudaError_t e1 = cudaSuccess;
-      for (int q = 0; q < b->graph_chunk && e1 == cudaSuccess; q++) e1 = enqueue_batch_step(b);
+      for (int q = 0; q < b->graph_chunk && e1 == cudaSuccess; q++) e1 = enqueue_batch_step(b, q);
+      if (e1 == cudaSuccess && b->rec_pending) e1 = cudaStreamWaitEvent(b->stream, b->rec_side.join, 0);
+      b->rec_pending = false;
+      if (e1 == cudaSuccess) e1 = launch_batch_advance(b->d_rp, (int)b->cases.size(), b->graph_chunk, b->stream);
       e = cudaStreamEndCapture(b->stream, &graph);
       if (e1 != cudaSuccess) return bcuda(b, e1, "kernel launch during capture");
       if (e != cudaSuccess) return bcuda(b, e, "cudaStreamEndCapture");
@@ -256,7 +283,7 @@ extern "C" int simb_run(simb_t *b, int nsteps) {
     }
   }
   for (; left > 0; left--)
-    if ((e = enqueue_batch_step(b)) != cudaSuccess) return bcuda(b, e, "kernel launch");
+    if ((e = enqueue_batch_step(b, -1)) != cudaSuccess) return bcuda(b, e, "kernel launch");
   b->steps_done += nsteps;
   for (sim_t *h : b->cases) sim_advance(h, nsteps);
   return SIM_OK;

@@ -50,11 +50,12 @@ struct KParams {
   const float *wav;     // [n_wav] stress increment of the source at step n (scaled)
   int n_wav;
   int src_i, src_j, src_k;  // src_j < 0: all ring-0 cells
-  int *step;                // device step counter
+  int *step;                // device step counter: the step is *step + step_off
   int i_lo, i_hi;           // rows updated: i_lo <= i < i_hi (the rest are interface ghost rows)
   // z cells the split kernels update: k_lo <= k < k_hi (a z slab's own cells;
   // the rest are its ghost cells, filled by the neighbouring slabs)
   int k_lo = 0, k_hi = 1 << 30;
+  int step_off = 0;  // of this launch's step from the counter (the steps of a captured chunk: 0, 1, ...)
 };
 
 // Point forces and the torsion ring (source kinds 1-3): entry e adds
@@ -69,6 +70,7 @@ struct IParams {
   const float *wav;
   int n_wav;
   int *step;
+  int step_off;
   void *f[NF];
 };
 
@@ -86,6 +88,7 @@ struct WParams {
   const float2 *m_lam;
   double iv2, is2;  // 1 / (storage scale)^2 of the velocities and the stresses
   int *step, *status;
+  int step_off;  // steps done = *step + step_off
   double *acc;
 };
 
@@ -250,7 +253,10 @@ struct PassParams {
 // launchers implemented in the .cu files (host side)
 // parts: 1 = velocity kernel, 2 = stress kernel, 3 = both (velocity first)
 cudaError_t launch_split(int storage, const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts = 3);
-cudaError_t launch_receivers(int storage, const RParams &p, cudaStream_t s);
+// receivers of the step *step + off; advance: the counter goes on by one (a
+// captured chunk counts by off instead and advances at its end)
+cudaError_t launch_receivers(int storage, const RParams &p, int off, bool advance, cudaStream_t s);
+cudaError_t launch_advance(int *step, int by, cudaStream_t s);
 cudaError_t launch_inject(int storage, const IParams &p, cudaStream_t s);
 cudaError_t launch_fused(int storage, int rt, const FusedMaps &maps, const FusedParams &fp, cudaStream_t s);
 size_t fused_smem_bytes(int storage, int rt);
@@ -260,7 +266,8 @@ size_t fused_smem_bytes(int storage, int rt);
 constexpr int BATCH_MAX = 64;
 long long batch_blocks(const KParams &p);
 cudaError_t launch_batch_split(int storage, bool vel, const KParams *cases, int n_cases, cudaStream_t s);
-cudaError_t launch_batch_receivers(int storage, const RParams *rp, int n_cases, cudaStream_t s);
+cudaError_t launch_batch_receivers(int storage, const RParams *rp, int n_cases, int off, bool advance, cudaStream_t s);
+cudaError_t launch_batch_advance(const RParams *rp, int n_cases, int by, cudaStream_t s);
 
 // Azimuthally refined grid: ghost rows filled from the neighbouring zone's
 // row through a dense [n_out][n_in] interpolation matrix along theta, for

@@ -276,7 +276,7 @@ __device__ __forceinline__ void sr_store(half_sr *p, const float (&v)[NV], const
 // the key of a body's stores: the step and the cell group (stochastic rounding only)
 template <typename T>
 __device__ __forceinline__ SrKey body_key(const KParams &p, int j, int i, int k0) {
-  if constexpr (std::is_same<T, half_sr>::value) return sr_key(p, *p.step, j, i, k0);
+  if constexpr (std::is_same<T, half_sr>::value) return sr_key(p, *p.step + p.step_off, j, i, k0);
   else return SrKey{0ull, 0ull, 0};
 }
 
@@ -666,7 +666,7 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
   }
   float src[NV] = {};
   if (i == p.src_i && (p.src_j < 0 || p.src_j == j) && p.src_k >= k0 && p.src_k < k0 + NV) {
-    const int n = *p.step;
+    const int n = *p.step + p.step_off;
     src[p.src_k - k0] = n < p.n_wav ? __ldg(p.wav + n) : 0.f;
   }
 

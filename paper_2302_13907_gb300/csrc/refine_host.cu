@@ -55,6 +55,9 @@ struct simr_s {
   static constexpr int MAX_ZSTREAMS = 7;
   cudaStream_t zs[MAX_ZSTREAMS] = {};
   cudaEvent_t zfork = nullptr, zjoin[MAX_ZSTREAMS] = {};
+  // captured chunks: the receivers of a step run beside the next one's velocities
+  SideStream rec_side{};
+  bool rec_pending = false;
   int big_zone = 0;
   bool zone_streams = false, forced = false;  // forced: opts.tile names the split codes
   int vel_code = 0, str_code = 0;  // split codes of every zone's halves
@@ -121,6 +124,9 @@ void rrelease(simr_t *h) {
     if (h->zjoin[k]) cudaEventDestroy(h->zjoin[k]);
   }
   if (h->zfork) cudaEventDestroy(h->zfork);
+  if (h->rec_side.fork) cudaEventDestroy(h->rec_side.fork);
+  if (h->rec_side.join) cudaEventDestroy(h->rec_side.join);
+  if (h->rec_side.side) cudaStreamDestroy(h->rec_side.side);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
@@ -180,17 +186,29 @@ cudaError_t zones_half(simr_t *h, int code, int parts) {
   return e;
 }
 
-cudaError_t enqueue_refined_step(simr_t *h) {
+// off >= 0: step `off` of a captured chunk, the receivers beside the next step's
+// velocities (see enqueue_step of the uniform grid); off < 0: a step by itself
+cudaError_t enqueue_refined_step(simr_t *h, int off) {
   cudaError_t e = cudaSuccess;
+  IParams ip = h->ip;
+  ip.step_off = std::max(off, 0);
+  for (KParams &p : h->kps) p.step_off = std::max(off, 0);
   const bool force = h->src_kind == 1 || h->src_kind == 2;
   e = zones_half(h, h->vel_code, 1);
-  if (e == cudaSuccess && force) e = launch_inject(0, h->ip, h->stream);
+  if (e == cudaSuccess && force) e = launch_inject(0, ip, h->stream);
   if (e == cudaSuccess) e = launch_xfer(h->xv, h->stream);
+  if (e == cudaSuccess && h->rec_pending) e = cudaStreamWaitEvent(h->stream, h->rec_side.join, 0);
   if (e == cudaSuccess) e = zones_half(h, h->str_code, 2);
-  if (e == cudaSuccess && h->src_kind == 3) e = launch_inject(0, h->ip, h->stream);
+  if (e == cudaSuccess && h->src_kind == 3) e = launch_inject(0, ip, h->stream);
   if (e == cudaSuccess) e = launch_xfer(h->xs, h->stream);
-  if (e == cudaSuccess) e = launch_batch_receivers(0, h->d_rp, (int)h->kps.size(), h->stream);
-  return e;
+  const int n = (int)h->kps.size();
+  if (e != cudaSuccess || off < 0)
+    return e != cudaSuccess ? e : launch_batch_receivers(0, h->d_rp, n, 0, true, h->stream);
+  if ((e = cudaEventRecord(h->rec_side.fork, h->stream)) != cudaSuccess) return e;
+  if ((e = cudaStreamWaitEvent(h->rec_side.side, h->rec_side.fork, 0)) != cudaSuccess) return e;
+  if ((e = launch_batch_receivers(0, h->d_rp, n, off, false, h->rec_side.side)) != cudaSuccess) return e;
+  h->rec_pending = true;
+  return cudaEventRecord(h->rec_side.join, h->rec_side.side);
 }
 
 }  // namespace
@@ -528,6 +546,10 @@ extern "C" int simr_create(const sim_grid_t *grid, const simr_zones_t *zones, co
     }
     if (M > 1 && (e = cudaEventCreateWithFlags(&h->zfork, cudaEventDisableTiming)) != cudaSuccess)
       return bail(rcuda(h, e, "zone streams"));
+    if ((e = cudaStreamCreateWithFlags(&h->rec_side.side, cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&h->rec_side.fork, cudaEventDisableTiming)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&h->rec_side.join, cudaEventDisableTiming)) != cudaSuccess)
+      return bail(rcuda(h, e, "receivers' stream"));
   }
   // the zones' split codes; a forced one is tried once per half on the still
   // zero state of zone 0 with the source off (the state stays zero)
@@ -697,7 +719,10 @@ extern "C" int simr_step(simr_t *h, int nsteps) {
       if ((e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
         return rcuda(h, e, "cudaStreamBeginCapture");
       cudaError_t e1 = cudaSuccess;
-      for (int q = 0; q < h->graph_chunk && e1 == cudaSuccess; q++) e1 = enqueue_refined_step(h);
+      for (int q = 0; q < h->graph_chunk && e1 == cudaSuccess; q++) e1 = enqueue_refined_step(h, q);
+      if (e1 == cudaSuccess && h->rec_pending) e1 = cudaStreamWaitEvent(h->stream, h->rec_side.join, 0);
+      h->rec_pending = false;
+      if (e1 == cudaSuccess) e1 = launch_batch_advance(h->d_rp, (int)h->kps.size(), h->graph_chunk, h->stream);
       e = cudaStreamEndCapture(h->stream, &graph);
       if (e1 != cudaSuccess) return rcuda(h, e1, "kernel launch during capture");
       if (e != cudaSuccess) return rcuda(h, e, "cudaStreamEndCapture");
@@ -712,7 +737,7 @@ extern "C" int simr_step(simr_t *h, int nsteps) {
     }
   }
   for (; left > 0; left--)
-    if ((e = enqueue_refined_step(h)) != cudaSuccess) return rcuda(h, e, "kernel launch");
+    if ((e = enqueue_refined_step(h, -1)) != cudaSuccess) return rcuda(h, e, "kernel launch");
   h->steps_done += nsteps;
   return SIM_OK;
 }

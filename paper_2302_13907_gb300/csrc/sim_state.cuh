@@ -69,6 +69,10 @@ struct sim_s {
   RParams rp2[2];
   // second stream and fork / join events of the three-way split halves
   SideStream side{};
+  // captured chunks: the receivers of a step run beside the next step's first
+  // half (fork: the step is done; join: its samples are taken)
+  SideStream rec_side{};
+  bool rec_pending = false;
   // device watchdog (opts.watchdog_every > 0): parameters per step parity
   // (the fused path's state alternates between the buffer sets)
   int watch_every = 0, watch_blocks = 0;

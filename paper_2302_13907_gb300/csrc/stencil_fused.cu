@@ -313,7 +313,7 @@ __device__ __forceinline__ void fused_tile(const FusedMaps &maps, const FusedPar
             const float2 ll = __ldg(m_lam + Im[xi]);  // {lambda, lambda + 2 mu}
             float src = 0.f;
             if (i == p.src_i && k == p.src_k && (p.src_j < 0 || p.src_j == plane)) {
-              const int n = *p.step;
+              const int n = *p.step + p.step_off;
               src = n < p.n_wav ? __ldg(p.wav + n) : 0.f;
             }
             o[0] += dts * (ll.y * err + ll.x * (epp + ezz)) + src;

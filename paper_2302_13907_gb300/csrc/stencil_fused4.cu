@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(F4Smem<T, RT>::NT) fused4_step(const __grid_co
           const float2 ll = __ldg(m_lam + im[e]);
           float src = 0.f;
           if (i == p.src_i && k == p.src_k && (p.src_j < 0 || p.src_j == plane)) {
-            const int n = *p.step;
+            const int n = *p.step + p.step_off;
             src = n < p.n_wav ? __ldg(p.wav + n) : 0.f;
           }
           o[0][e] += dts * (ll.y * err + ll.x * (epp + ezz)) + src;

@@ -254,7 +254,7 @@ __device__ __forceinline__ void str_quad(const KParams &p, const unsigned char *
   const bool zl = pz > 0 && (kq < pz || kq + 3 >= NZ - pz);
   float src[4] = {0.f, 0.f, 0.f, 0.f};
   if (i == p.src_i && (p.src_j < 0 || p.src_j == j) && p.src_k >= kq && p.src_k < kq + 4) {
-    const int n = *p.step;
+    const int n = *p.step + p.step_off;
     src[p.src_k - kq] = n < p.n_wav ? __ldg(p.wav + n) : 0.f;
   }
 

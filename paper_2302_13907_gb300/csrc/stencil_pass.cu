@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(PassSmem<R>::WARPS * 32, 1)
           }
         }
         if (force_cell) {  // point force (v_r or v_z), on the recomputed halo as well
-          const int st = *p.step, jj = j >= nth ? j - nth : j;
+          const int st = *p.step + p.step_off, jj = j >= nth ? j - nth : j;
           const float w = st < p.n_wav ? __ldg(q.force_w + jj) * __ldg(q.force_wav + st) : 0.f;
 #pragma unroll
           for (int e = 0; e < 4; e++)
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(PassSmem<R>::WARPS * 32, 1)
             opz[e] += dts4 * rcp_fast(sjc[e] + sjc[e + 1]) * (Q + gz);
           }
           if (src_cell && (p.src_j < 0 || p.src_j == j - 1)) {
-            const int st = *p.step;
+            const int st = *p.step + p.step_off;
             const float w = st < p.n_wav ? __ldg(p.wav + st) : 0.f;
 #pragma unroll
             for (int e = 0; e < 4; e++)

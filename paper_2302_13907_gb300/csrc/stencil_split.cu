@@ -217,7 +217,7 @@ __device__ __forceinline__ void str_body(const KParams &p, const int j, const in
   // source: step-indexed increment of the three normal stresses
   float src[4] = {0.f, 0.f, 0.f, 0.f};
   if (i == p.src_i && (p.src_j < 0 || p.src_j == j) && p.src_k >= k0 && p.src_k < k0 + 4) {
-    const int n = *p.step;
+    const int n = *p.step + p.step_off;
     src[p.src_k - k0] = n < p.n_wav ? __ldg(p.wav + n) : 0.f;
   }
 
@@ -355,10 +355,10 @@ __global__ void __launch_bounds__(SB_X *SB_Y, SB_MINB) str_split(const KParams p
 
 
 // Pressure at the receivers after the stress update; one block, fixed
-// summation order over theta; advances the device step counter.
+// summation order over theta; advances the device step counter if asked to.
 template <typename T>
-__device__ __forceinline__ void receivers_body(const RParams &p) {
-  const int n = *p.step;
+__device__ __forceinline__ void receivers_body(const RParams &p, int off, bool advance) {
+  const int n = *p.step + off;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const T *srr = (const T *)p.srr, *spp = (const T *)p.spp, *szz = (const T *)p.szz;
   for (int r = warp; r < p.n_rec; r += blockDim.x >> 5) {
@@ -381,6 +381,7 @@ __device__ __forceinline__ void receivers_body(const RParams &p) {
       if (n < p.cap) p.traces[(long long)r * p.cap + n] = v;
     }
   }
+  if (!advance) return;
   __syncthreads();
   if (threadIdx.x == 0) *p.step = n + 1;
 }
@@ -400,22 +401,25 @@ template <typename T>
 __global__ void __launch_bounds__(128) inject_kernel(const IParams p) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= p.n) return;
-  const int n = *p.step;
+  const int n = *p.step + p.step_off;
   if (n < 0 || n >= p.n_wav) return;
   T *x = (T *)p.f[p.fld[e]] + p.off[e];
   *x = to_store<T>(st_to_float<T>(*x) + p.w[e] * __ldg(p.wav + n));
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) receivers_kernel(const RParams p) {
-  receivers_body<T>(p);
+__global__ void __launch_bounds__(256) receivers_kernel(const RParams p, int off, bool advance) {
+  receivers_body<T>(p, off, advance);
 }
 
 // one block per case
 template <typename T>
-__global__ void __launch_bounds__(256) receivers_batch(const RParams *rp) {
-  receivers_body<T>(rp[blockIdx.x]);
+__global__ void __launch_bounds__(256) receivers_batch(const RParams *rp, int off, bool advance) {
+  receivers_body<T>(rp[blockIdx.x], off, advance);
 }
+
+__global__ void advance_kernel(int *step, int by) { *step += by; }
+__global__ void advance_batch(const RParams *rp, int by) { *rp[blockIdx.x].step += by; }
 
 template <typename T>
 static cudaError_t launch_split_t(const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts) {
@@ -442,11 +446,11 @@ cudaError_t launch_split(int storage, const KParams &p, cudaStream_t s, cudaEven
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_batch_receivers(int storage, const RParams *rp, int n_cases, cudaStream_t s) {
+cudaError_t launch_batch_receivers(int storage, const RParams *rp, int n_cases, int off, bool advance, cudaStream_t s) {
   switch (storage) {
-    case 0: receivers_batch<float><<<n_cases, 256, 0, s>>>(rp); break;
-    case 1: receivers_batch<__nv_bfloat16><<<n_cases, 256, 0, s>>>(rp); break;
-    case 2: receivers_batch<__half><<<n_cases, 256, 0, s>>>(rp); break;
+    case 0: receivers_batch<float><<<n_cases, 256, 0, s>>>(rp, off, advance); break;
+    case 1: receivers_batch<__nv_bfloat16><<<n_cases, 256, 0, s>>>(rp, off, advance); break;
+    case 2: receivers_batch<__half><<<n_cases, 256, 0, s>>>(rp, off, advance); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -464,11 +468,21 @@ cudaError_t launch_inject(int storage, const IParams &p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_receivers(int storage, const RParams &p, cudaStream_t s) {
+cudaError_t launch_advance(int *step, int by, cudaStream_t s) {
+  advance_kernel<<<1, 1, 0, s>>>(step, by);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_advance(const RParams *rp, int n_cases, int by, cudaStream_t s) {
+  advance_batch<<<n_cases, 1, 0, s>>>(rp, by);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_receivers(int storage, const RParams &p, int off, bool advance, cudaStream_t s) {
   switch (storage) {
-    case 0: receivers_kernel<float><<<1, 256, 0, s>>>(p); break;
-    case 1: receivers_kernel<__nv_bfloat16><<<1, 256, 0, s>>>(p); break;
-    case 2: receivers_kernel<__half><<<1, 256, 0, s>>>(p); break;
+    case 0: receivers_kernel<float><<<1, 256, 0, s>>>(p, off, advance); break;
+    case 1: receivers_kernel<__nv_bfloat16><<<1, 256, 0, s>>>(p, off, advance); break;
+    case 2: receivers_kernel<__half><<<1, 256, 0, s>>>(p, off, advance); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -34,7 +34,7 @@ __device__ __forceinline__ double ld(const void *f, long long c) {
 
 template <typename T>
 __global__ void __launch_bounds__(WATCH_THREADS) watch_reduce(const WParams p) {
-  const int n = *p.step;
+  const int n = *p.step + p.step_off;
   if (n % p.every != 0) return;  // the same for every block
   const long long rows = (long long)p.nth * p.NR;
   double acc = 0.0;
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(WATCH_THREADS) watch_reduce(const WParams p) {
 
 // one thread: the decision on the sum the reduction left in acc[0]
 __global__ void watch_check(const WParams p) {
-  const int n = *p.step;
+  const int n = *p.step + p.step_off;
   if (n % p.every != 0) return;
   double *a = p.acc;
   const double E = a[0];
