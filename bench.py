@@ -91,7 +91,8 @@ def kernel_hash() -> str:
     csrc = os.path.join(ROOT, "paper_2302_13907_gb300", "csrc")
     files = glob.glob(os.path.join(csrc, "stencil_*.cu")) + [os.path.join(csrc, "cwell_internal.cuh"),
                                                              os.path.join(csrc, "tma_util.cuh"),
-                                                             os.path.join(csrc, "hoist_body.cuh")]
+                                                             os.path.join(csrc, "hoist_body.cuh"),
+                                                             os.path.join(csrc, "hoist_run.cuh")]
     for f in sorted(f for f in files if os.path.basename(f) != "stencil_refine.cu"):
         code = re.sub(r"/\*.*?\*/", " ", open(f).read(), flags=re.S)
         code = re.sub(r"//[^\n]*", " ", code)

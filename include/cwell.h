@@ -283,11 +283,13 @@ size_t sim_device_bytes(const sim_t *h);
  * blocks/SM), 2 (two cells, both in one launch), 3 (two, 6), 4 (four, 3);
  * interior two cells, b = 6, 8, with edge c = 1 (two, 6) or 5 (two; b = 6 in one
  * launch, b = 8 edge for 4 blocks/SM); c = 6, 7: edge (two, 4), (four, 3) with a
- * persistent interior kernel prefetching its next tile into L2; c = 8 as 4 and
+ * persistent interior kernel prefetching its next tile into L2 (2275: the
+ * interior marched along theta, the edge of c = 8); c = 8 as 4 and
  * c = 9 as 6, each with the radial tiles walked the same way; 2300 + 10 c + b
  * for a three-way split (interior; radial-PML rows; z ends), interior b = 5
  * plain or 4 prefetching, c = 0 to 3 the radial / end kernels' cells per thread
- * and blocks per SM;
+ * and blocks per SM (2324: the interior and, in FP32, the radial layer marched
+ * along theta);
  * v * 10000 + s (a pair code) for the velocity kernel of split code v with the
  * stress kernel of split code s; 3000 + 100 m + 10 e + b for the single-pass
  * sweep kernel (kernel = SIM_KERNEL_SWEEP: four z cells per thread, b resident
@@ -301,7 +303,8 @@ size_t sim_device_bytes(const sim_t *h);
  * materials; SIM_EINVAL otherwise): both halves of the lean cells in one kernel,
  * theta in d runs (1 .. nth, at most 32) per tile, m = 0, 2: one block per SM
  * walks the tiles, 1, 3: one block per tile; the other cells with split bodies of
- * two (m = 0, 1) or four (2, 3) cells per thread.
+ * two (m = 0, 1) or four (2, 3; the radial layer marched along theta) cells per
+ * thread.
  * opts.tile accepts every code listed here. */
 int sim_config(const sim_t *h, int *kernel, int *tile_rows);
 
@@ -399,8 +402,8 @@ const char *simb_last_error(const simb_t *b);
  * rows per zone, the radial PML inside the last zone (row0 <= nr - 2); FP32
  * storage; any source kind, placed on the nodes of the zone that holds it
  * (the transverse force off the axis and the torsion ring not on a zone's
- * first row, SIM_EUNSUPPORTED).  Every zone runs the split kernels, velocity
- * code 2285 and stress code 2334 (largest zone of at least 8 Mi cells; the
+ * first row, SIM_EUNSUPPORTED).  Every zone runs the split kernels, code
+ * 2324 (largest zone of at least 8 Mi cells; the
  * zones of a half then run on parallel streams); on smaller grids all zones of
  * a half share one launch.  opts.tile may name a 22xx / 23xx split code or pair
  * code instead (SIM_EINVAL otherwise; small grids then run zone after zone).

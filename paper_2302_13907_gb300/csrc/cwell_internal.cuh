@@ -56,6 +56,7 @@ struct KParams {
   // the rest are its ghost cells, filled by the neighbouring slabs)
   int k_lo = 0, k_hi = 1 << 30;
   int step_off = 0;  // of this launch's step from the counter (the steps of a captured chunk: 0, 1, ...)
+  int n_mat = 0;
 };
 
 // Point forces and the torsion ring (source kinds 1-3): entry e adds
@@ -315,13 +316,15 @@ size_t march_smem_bytes(int storage, int code);
 // blocks per SM; c = 3: two cells, 6 blocks; c = 4: four cells, 3 blocks; c = 5:
 // two cells in both, b = 6: one launch for 5 blocks per SM, b = 8: interior for
 // 8, edge for 4; c = 6 / 7: two cells, 4 blocks / four cells, 3 blocks with a
-// persistent interior kernel that prefetches its next tile into L2; c = 8: plain
+// persistent interior kernel that prefetches its next tile into L2 (2275: with the
+// interior marched along theta, hoist_run.cuh, and the edge of c = 8); c = 8: plain
 // interior, edge (four cells, 3 blocks) whose radial tiles are walked with the
 // same prefetch; c = 9: prefetching interior and prefetching edge (two cells, 4
 // blocks); 2300 + 10 c + b = three-way split (interior, radial-PML rows, z ends;
 // the radial kernel persistent and prefetching): interior b = 5 plain, 4
 // prefetching, and c = 0: radial (four cells, 4 blocks per SM) + ends (four, 3);
-// 1: (two, 5) + (two, 4); 2: (two, 4) + (two, 4); 3: (four, 3) + (four, 3).  A
+// 1: (two, 5) + (two, 4); 2: (two, 4) + (two, 4); 3: (four, 3) + (four, 3); 2324:
+// interior and, in FP32, radial layer marched along theta, the rest as c = 3.  A
 // pair code v * 10000 + s runs the velocity kernel of split code v and the
 // stress kernel of split code s (the autotuner times the two apart).
 constexpr int SPLIT_CODE = 2000;
@@ -355,7 +358,7 @@ void set_side_stream(const SideStream *ss);
 // one-pass step: tile code 4000 + 100 m + d, theta cut into d runs per tile;
 // m odd: one block per item, even: one block per SM walks them; m = 0, 1: the
 // split bodies on the rest of the cells take two cells per thread, m = 2, 3:
-// four.  launch_pass_edges: PASS_VEL = their velocities and PASS_STR_LAYER = the
+// four (the radial layer marched along theta).  launch_pass_edges: PASS_VEL = their velocities and PASS_STR_LAYER = the
 // stresses that need no velocity of the pass (the radial layer but its rim
 // row), both beside the pass; PASS_STR_RIM = the other stresses, after both.
 inline bool is_pass(int code) { return code > 4000 && code < 4400 && code % 100 >= 1 && code % 100 <= 32; }

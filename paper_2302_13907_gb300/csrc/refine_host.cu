@@ -141,12 +141,12 @@ double dirichlet(int N, double t) {
 bool pow2_in(int n) { return n == 4 || n == 8 || n == 16 || n == 32 || n == 64; }
 
 // split codes of a grid whose largest zone fills the GPU (the 20 m well; the
-// zones then run on parallel streams), the fastest pair measured: plain
-// interior + prefetching edge for the velocities, the three-way split for the
-// stresses.  A smaller grid (a 1.6 m crop, several handles side by side) runs
+// zones then run on parallel streams): interior and radial layer marched along
+// theta, 1375 us a step of the 20 m well where the best tile-by-tile pair (2285 and
+// 2334) takes 1449.  A smaller grid (a 1.6 m crop, several handles side by side) runs
 // all zones of a half in one launch of the batched kernel: 126 us a step of the
 // 136 x 32 x 1330 crop, 176 with two launches per zone and half.
-constexpr int REFINED_VEL_CODE = 2285, REFINED_STR_CODE = 2334;
+constexpr int REFINED_VEL_CODE = 2324, REFINED_STR_CODE = 2324;
 constexpr long long ZONE_STREAM_CELLS = 8LL << 20;
 // opts.tile of a refined handle: 0, or a split code or pair code whose halves
 // are interior / edge (22xx) or three-way (23xx) split codes
@@ -499,6 +499,7 @@ extern "C" int simr_create(const sim_grid_t *grid, const simr_zones_t *zones, co
     p.ab_q = Z.ab_q;
     p.ab_z = h->ab_z;
     p.mat = h->mat;
+    p.n_mat = medium->n_mat;
     p.m_rho = h->m_rho;
     p.m_imu = h->m_imu;
     p.m_lam = h->m_lam;

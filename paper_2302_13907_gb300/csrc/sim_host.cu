@@ -904,6 +904,7 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
   p.ab_q = h->ab_q;
   p.ab_z = h->ab_z;
   p.mat = h->mat;
+  p.n_mat = h->n_mat;
   p.m_rho = h->m_rho;
   p.m_imu = h->m_imu;
   p.m_lam = h->m_lam;

@@ -9,7 +9,7 @@
 // launches (a lean-only kernel on the interior tiles).
 #include <algorithm>
 
-#include "hoist_body.cuh"
+#include "hoist_run.cuh"
 
 namespace cwell {
 namespace {
@@ -167,6 +167,39 @@ __global__ void __launch_bounds__(HB_X *HB_Y, MINB) hoist_interior_pf(const KPar
     if (t + (int)gridDim.x < n && interior_cell<NV>(p, q, t + gridDim.x, j, i, k0)) prefetch_tile<T, NV, VEL>(p, j, i, k0);
     if (interior_cell<NV>(p, q, t, j, i, k0)) lean_cells_step<T, NV, VEL>(p, j, i, k0);
   }
+}
+
+// tiles of the interior (RAD: of the radial layer) marched along theta in runs of
+// `run` planes (last run shorter); block = one tile of one run, z tiles fastest,
+// then r, then the runs; OUT: out of place into `set`
+template <typename T, int MINB, bool VEL, bool RAD, bool OUT = false>
+__global__ void __launch_bounds__(HB_X *HB_Y, MINB) hoist_run(const KParams p, const Regions q, int run, const OutSet set) {
+  extern __shared__ float2 run_tab[];
+  run_table<VEL>(p, run_tab);
+  const int nzt = RAD ? q.rnzt : q.nzt, nrt = RAD ? q.rnrt : q.nrt;
+  int t = blockIdx.x;
+  const int k0 = (((RAD ? q.rzt0 : q.zt0) + t % nzt) * HB_X + threadIdx.x) * 4;
+  t /= nzt;
+  const int i = (RAD ? q.r0 : p.i_lo) + (t % nrt) * HB_Y + threadIdx.y, j0 = t / nrt * run, J = min(run, p.nth - j0);
+  const bool in = RAD ? i >= p.i_lo : i < q.r0;
+  if (!(in && i < p.i_hi && k0 >= q.za && k0 < q.zb && k0 >= p.k_lo && k0 < p.k_hi)) return;
+  void *const *fo = OUT ? set.f : p.f;
+  if (VEL) vel_run<T, RAD>(p, fo, (const float *)run_tab, j0, J, i, k0);
+  else str_run<T, RAD>(p, fo, run_tab, (const float *)(run_tab + p.n_mat), j0, J, i, k0);
+}
+
+// planes per run: the fewest rounds of resident blocks times the planes each
+// passes over (a run loads about one plane's worth before its first)
+inline int run_planes(long long tiles, int nth, int slots) {
+  int best = nth;
+  double cost = 1e300;
+  for (int d = 1; d <= std::max(1, nth / 4); d++) {
+    const int run = (nth + d - 1) / d;
+    const long long items = tiles * ((nth + run - 1) / run);
+    const double c = (double)((items + slots - 1) / slots) * (run + 1);
+    if (c < cost) cost = c, best = run;
+  }
+  return best;
 }
 
 // L2 prefetch of a radial-layer tile: the fields' rows and the memory variables
@@ -354,10 +387,30 @@ inline cudaError_t side_join(bool fork, cudaStream_t s) {
 
 inline int wave(long long tiles, int minb) { return (int)std::min<long long>(tiles, (long long)sm_count() * minb); }
 
-template <typename T, int NV, int MINB, bool PF, bool VEL>
+// tables and arrays beyond the march's shared memory and 32-bit offsets go tile by tile
+template <typename T>
+bool can_run(const KParams &p) {
+  const unsigned long long lim = 0xffffffffull - 4096;
+  return p.n_mat <= RUN_MATS && (unsigned long long)p.plane * p.nth * sizeof(T) < lim &&
+         (unsigned long long)p.pml_r * p.NZp * p.nth * 4 < lim;
+}
+template <typename T, int MINB, bool VEL, bool RAD, bool OUT>
+void launch_run(const KParams &p, const Regions &q, const OutSet &set, cudaStream_t s) {
+  const int tiles = RAD ? q.rnrt * q.rnzt : q.nrt * q.nzt, run = run_planes(tiles, p.nth, sm_count() * MINB);
+  hoist_run<T, MINB, VEL, RAD, OUT><<<tiles * ((p.nth + run - 1) / run), dim3(HB_X, HB_Y),
+                                      run_table_bytes(p.n_mat, VEL), s>>>(p, q, run, set);
+}
+
+// MODE 0: one tile per block; 1: persistent with prefetch; 2: marched along theta
+template <typename T, int NV, int MINB, int MODE, bool VEL>
 void launch_interior(const KParams &p, const Regions &q, cudaStream_t s) {
   dim3 blk(HB_X, HB_Y);
-  if constexpr (PF) hoist_interior_pf<T, NV, MINB, VEL><<<wave(q.interior, MINB), blk, 0, s>>>(p, q);
+  if constexpr (MODE == 2) {
+    static_assert(NV == 4, "four cells per thread");
+    constexpr int MB = sizeof(T) == 2 && !VEL ? MINB - 1 : MINB;  // without spills: 3 stress blocks, 4 velocity blocks
+    if (can_run<T>(p)) launch_run<T, MB, VEL, false, false>(p, q, OutSet{}, s);
+    else hoist_interior<T, NV, 4, VEL><<<(int)q.interior, blk, 0, s>>>(p, q);
+  } else if constexpr (MODE == 1) hoist_interior_pf<T, NV, MINB, VEL><<<wave(q.interior, MINB), blk, 0, s>>>(p, q);
   else hoist_interior<T, NV, MINB, VEL><<<(int)q.interior, blk, 0, s>>>(p, q);
 }
 
@@ -365,7 +418,7 @@ void launch_interior(const KParams &p, const Regions &q, cudaStream_t s) {
 // (g_side): the regions update disjoint cells from inputs no launch of the half
 // writes.  MINB_R = 0: one edge launch (22xx); otherwise the radial layer
 // (MINB_R blocks per SM) and the z ends apart (23xx).
-template <typename T, int NV, int MINB_IN, bool PF, int NVE, int MINB_R, int MINB_E, bool PFE, bool VEL>
+template <typename T, int NV, int MINB_IN, int MODE, int NVE, int MINB_R, int MINB_E, int PFE, bool VEL>
 cudaError_t launch_split_half(const KParams &p, const Regions &q, cudaStream_t s) {
   dim3 blk(HB_X, HB_Y);
   const bool edge = q.radial > 0 || q.ends > 0;
@@ -374,13 +427,20 @@ cudaError_t launch_split_half(const KParams &p, const Regions &q, cudaStream_t s
   cudaError_t e = side_fork(fork, s, &se);
   if (e != cudaSuccess) return e;
   if constexpr (MINB_R == 0) {
-    const int rad = PFE ? wave(q.radial, MINB_E) : (int)q.radial;
-    if (edge) hoist_edge<T, NVE, MINB_E, VEL, PFE><<<(int)q.ends + rad, blk, 0, se>>>(p, q, OutSet{});
+    const int rad = PFE ? wave(q.radial, PFE) : (int)q.radial;
+    if (edge) hoist_edge<T, NVE, MINB_E, VEL, (PFE > 0)><<<(int)q.ends + rad, blk, 0, se>>>(p, q, OutSet{});
   } else {
-    if (q.radial > 0) hoist_radial_pf<T, NVE, MINB_R, VEL><<<wave(q.radial, MINB_R), blk, 0, se>>>(p, q);
+    if (q.radial > 0) {
+      if constexpr (MODE == 2 && sizeof(T) == 4) {
+        if (can_run<T>(p)) launch_run<T, 2, VEL, true, false>(p, q, OutSet{}, se);
+        else hoist_radial_pf<T, NVE, MINB_R, VEL><<<wave(q.radial, MINB_R), blk, 0, se>>>(p, q);
+      } else {
+        hoist_radial_pf<T, NVE, MINB_R, VEL><<<wave(q.radial, MINB_R), blk, 0, se>>>(p, q);
+      }
+    }
     if (q.ends > 0) hoist_ends<T, NVE, MINB_E, VEL><<<(int)q.ends, blk, 0, se>>>(p, q);
   }
-  if (q.interior > 0) launch_interior<T, NV, MINB_IN, PF, VEL>(p, q, s);
+  if (q.interior > 0) launch_interior<T, NV, MINB_IN, MODE, VEL>(p, q, s);
   if ((e = side_join(fork, s)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -388,19 +448,19 @@ cudaError_t launch_split_half(const KParams &p, const Regions &q, cudaStream_t s
 // block counts and the end threads' numbers are 32-bit
 inline bool fits(const Regions &q) { return q.interior + q.radial + q.ends * (HB_X * HB_Y) <= 0x7fffffffLL; }
 
-template <typename T, int NV, int MINB_IN, bool PF, int NVE, int MINB_R, int MINB_E, bool PFE = false>
+template <typename T, int NV, int MINB_IN, int MODE, int NVE, int MINB_R, int MINB_E, int PFE = 0>
 cudaError_t launch_split_t(const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts) {
   const Regions q = regions<NV, NVE>(p);
   if (!fits(q)) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
   if (parts & 1) {
     if (ev) cudaEventRecord(ev[0], s);
-    e = launch_split_half<T, NV, MINB_IN, PF, NVE, MINB_R, MINB_E, PFE, true>(p, q, s);
+    e = launch_split_half<T, NV, MINB_IN, MODE, NVE, MINB_R, MINB_E, PFE, true>(p, q, s);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], s);
   }
   if (parts & 2) {
-    e = launch_split_half<T, NV, MINB_IN, PF, NVE, MINB_R, MINB_E, PFE, false>(p, q, s);
+    e = launch_split_half<T, NV, MINB_IN, MODE, NVE, MINB_R, MINB_E, PFE, false>(p, q, s);
     if (ev) cudaEventRecord(ev[2], s);
   }
   return e;
@@ -442,7 +502,7 @@ cudaError_t launch_hoist_t(const KParams &p, cudaStream_t s, cudaEvent_t *ev, in
 }
 
 // the cells beside a one-pass step's: z ends, radial layer and its rim row r1
-template <int NV, int MINB>
+template <int NV, int MINB, bool RUN>
 cudaError_t launch_pass_edges_t(int part, const KParams &p, const OutSet &out, cudaStream_t s) {
   int r1, z0, z1;
   if (!pass_region(p, &r1, &z0, &z1)) return cudaErrorInvalidValue;
@@ -455,8 +515,13 @@ cudaError_t launch_pass_edges_t(int part, const KParams &p, const OutSet &out, c
     return cudaGetLastError();
   }
   if (part == PASS_STR_LAYER) q.ends = 0;
-  const int grid = (int)q.ends + wave(q.radial, MINB);
-  if (grid == 0) return cudaSuccess;
+  const bool march = RUN && q.radial > 0 && can_run<float>(p);
+  if (march) {
+    if (part == PASS_VEL) launch_run<float, 2, true, true, true>(p, q, out, s);
+    else launch_run<float, 2, false, true, true>(p, q, out, s);
+  }
+  const int grid = (int)q.ends + (march ? 0 : wave(q.radial, MINB));
+  if (grid == 0) return cudaGetLastError();
   if (part == PASS_VEL) hoist_edge<float, NV, MINB, true, true, true><<<grid, blk, 0, s>>>(p, q, out);
   else hoist_edge<float, NV, MINB, false, true, true><<<grid, blk, 0, s>>>(p, q, out);
   return cudaGetLastError();
@@ -466,14 +531,14 @@ cudaError_t launch_pass_edges_t(int part, const KParams &p, const OutSet &out, c
 template <typename T>
 cudaError_t launch_split3(int code, const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts) {
   switch (code) {
-    case 2304: return launch_split_t<T, 4, 4, true, 4, 4, 3>(p, s, ev, parts);
-    case 2305: return launch_split_t<T, 4, 5, false, 4, 4, 3>(p, s, ev, parts);
-    case 2314: return launch_split_t<T, 4, 4, true, 2, 5, 4>(p, s, ev, parts);
-    case 2315: return launch_split_t<T, 4, 5, false, 2, 5, 4>(p, s, ev, parts);
-    case 2324: return launch_split_t<T, 4, 4, true, 2, 4, 4>(p, s, ev, parts);
-    case 2325: return launch_split_t<T, 4, 5, false, 2, 4, 4>(p, s, ev, parts);
-    case 2334: return launch_split_t<T, 4, 4, true, 4, 3, 3>(p, s, ev, parts);
-    case 2335: return launch_split_t<T, 4, 5, false, 4, 3, 3>(p, s, ev, parts);
+    case 2304: return launch_split_t<T, 4, 4, 1, 4, 4, 3>(p, s, ev, parts);
+    case 2305: return launch_split_t<T, 4, 5, 0, 4, 4, 3>(p, s, ev, parts);
+    case 2314: return launch_split_t<T, 4, 4, 1, 2, 5, 4>(p, s, ev, parts);
+    case 2315: return launch_split_t<T, 4, 5, 0, 2, 5, 4>(p, s, ev, parts);
+    case 2324: return launch_split_t<T, 4, sizeof(T) == 4 ? 3 : 4, 2, 4, 3, 3>(p, s, ev, parts);
+    case 2325: return launch_split_t<T, 4, 5, 0, 2, 4, 4>(p, s, ev, parts);
+    case 2334: return launch_split_t<T, 4, 4, 1, 4, 3, 3>(p, s, ev, parts);
+    case 2335: return launch_split_t<T, 4, 5, 0, 4, 3, 3>(p, s, ev, parts);
   }
   return cudaErrorInvalidValue;
 }
@@ -488,26 +553,26 @@ cudaError_t launch_hoist_st(int code, const KParams &p, cudaStream_t s, cudaEven
     case 2005: return launch_hoist_t<T, 4, 5, false>(p, s, ev, parts);
     case 2106: return launch_hoist_t<T, 2, 6, false>(p, s, ev, parts);
     case 2108: return launch_hoist_t<T, 2, 8, false>(p, s, ev, parts);
-    case 2204: return launch_split_t<T, 4, 4, false, 4, 0, 4>(p, s, ev, parts);
-    case 2205: return launch_split_t<T, 4, 5, false, 4, 0, 4>(p, s, ev, parts);
-    case 2216: return launch_split_t<T, 2, 6, false, 2, 0, 6>(p, s, ev, parts);
-    case 2218: return launch_split_t<T, 2, 8, false, 2, 0, 6>(p, s, ev, parts);
+    case 2204: return launch_split_t<T, 4, 4, 0, 4, 0, 4>(p, s, ev, parts);
+    case 2205: return launch_split_t<T, 4, 5, 0, 4, 0, 4>(p, s, ev, parts);
+    case 2216: return launch_split_t<T, 2, 6, 0, 2, 0, 6>(p, s, ev, parts);
+    case 2218: return launch_split_t<T, 2, 8, 0, 2, 0, 6>(p, s, ev, parts);
     case 2224: return launch_one_t<T, 4, 2, 4>(p, s, ev, parts);
     case 2225: return launch_one_t<T, 4, 2, 5>(p, s, ev, parts);
-    case 2234: return launch_split_t<T, 4, 4, false, 2, 0, 6>(p, s, ev, parts);
-    case 2235: return launch_split_t<T, 4, 5, false, 2, 0, 6>(p, s, ev, parts);
-    case 2244: return launch_split_t<T, 4, 4, false, 4, 0, 3>(p, s, ev, parts);
-    case 2245: return launch_split_t<T, 4, 5, false, 4, 0, 3>(p, s, ev, parts);
+    case 2234: return launch_split_t<T, 4, 4, 0, 2, 0, 6>(p, s, ev, parts);
+    case 2235: return launch_split_t<T, 4, 5, 0, 2, 0, 6>(p, s, ev, parts);
+    case 2244: return launch_split_t<T, 4, 4, 0, 4, 0, 3>(p, s, ev, parts);
+    case 2245: return launch_split_t<T, 4, 5, 0, 4, 0, 3>(p, s, ev, parts);
     case 2256: return launch_one_t<T, 2, 2, 5>(p, s, ev, parts);
-    case 2258: return launch_split_t<T, 2, 8, false, 2, 0, 4>(p, s, ev, parts);
-    case 2264: return launch_split_t<T, 4, 4, true, 2, 0, 4>(p, s, ev, parts);
-    case 2265: return launch_split_t<T, 4, 5, true, 2, 0, 4>(p, s, ev, parts);
-    case 2274: return launch_split_t<T, 4, 4, true, 4, 0, 3>(p, s, ev, parts);
-    case 2275: return launch_split_t<T, 4, 5, true, 4, 0, 3>(p, s, ev, parts);
-    case 2284: return launch_split_t<T, 4, 4, false, 4, 0, 3, true>(p, s, ev, parts);
-    case 2285: return launch_split_t<T, 4, 5, false, 4, 0, 3, true>(p, s, ev, parts);
-    case 2294: return launch_split_t<T, 4, 4, true, 2, 0, 4, true>(p, s, ev, parts);
-    case 2295: return launch_split_t<T, 4, 5, true, 2, 0, 4, true>(p, s, ev, parts);
+    case 2258: return launch_split_t<T, 2, 8, 0, 2, 0, 4>(p, s, ev, parts);
+    case 2264: return launch_split_t<T, 4, 4, 1, 2, 0, 4>(p, s, ev, parts);
+    case 2265: return launch_split_t<T, 4, 5, 1, 2, 0, 4>(p, s, ev, parts);
+    case 2274: return launch_split_t<T, 4, 4, 1, 4, 0, 3>(p, s, ev, parts);
+    case 2275: return launch_split_t<T, 4, sizeof(T) == 4 ? 3 : 4, 2, 4, 0, 3, 3>(p, s, ev, parts);
+    case 2284: return launch_split_t<T, 4, 4, 0, 4, 0, 3, 3>(p, s, ev, parts);
+    case 2285: return launch_split_t<T, 4, 5, 0, 4, 0, 3, 3>(p, s, ev, parts);
+    case 2294: return launch_split_t<T, 4, 4, 1, 2, 0, 4, 4>(p, s, ev, parts);
+    case 2295: return launch_split_t<T, 4, 5, 1, 2, 0, 4, 4>(p, s, ev, parts);
   }
   return launch_split3<T>(code, p, s, ev, parts);
 }
@@ -551,7 +616,7 @@ cudaError_t launch_sr_round(const float *x, const unsigned *dither, unsigned sho
 }
 
 cudaError_t launch_pass_edges(int code, int part, const KParams &p, const OutSet &out, cudaStream_t s) {
-  return pass_edges4(code) ? launch_pass_edges_t<4, 3>(part, p, out, s) : launch_pass_edges_t<2, 4>(part, p, out, s);
+  return pass_edges4(code) ? launch_pass_edges_t<4, 3, true>(part, p, out, s) : launch_pass_edges_t<2, 4, false>(part, p, out, s);
 }
 
 cudaError_t launch_hoist(int storage, int code, const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts) {

@@ -45,3 +45,46 @@ def test_fields_at_region_edges(tile, nr, pml_r, nz, pml_z):
             b = o.field(n)
             assert np.abs(b).max() > 0, n
             assert np.abs(s.field(n) - b).max() <= 2e-5 * np.abs(b).max(), n
+
+
+@pytest.mark.parametrize("tile", [2275, 2324])
+@pytest.mark.parametrize("storage", ["f32", "bf16", "f16", "f16sr"])
+@pytest.mark.parametrize("nth,nr,pml_r,nz,pml_z,pml_on,n_mat", [
+    (10, 6, 1, 117, 2, True, 5),        # two runs of five planes, one z tile cut at both ends
+    (22, 5, 3, 146, 3, True, 2048),     # runs of five and a last one of two; the largest table in shared memory
+    (4, 7, 2, 252, 4, True, 2049),      # one run; a table that stays in L1
+    (6, 9, 0, 140, 0, False, 5),        # rigid walls: the last row has no outer neighbour
+])
+def test_march_along_theta(tile, storage, nth, nr, pml_r, nz, pml_z, pml_on, n_mat):
+    """The interior marched along theta against the tile-by-tile kernels, every
+    field: the same bits.  (Tile 2324 in FP32 marches the radial layer too, whose
+    products and sums may be fused differently: 2e-5 of the maximum.)"""
+    from paper_2302_13907_gb300.binding import Simulation
+    if storage == "f16sr" and tile < 2300:
+        pytest.skip("the stochastic rounding runs on the 23xx codes")
+    g = W.Grid(nr=nr, nth=nth, nz=nz, pml_r=pml_r, pml_z=pml_z, dr=0.004, dz=0.003)
+    rng = np.random.default_rng(nz)
+    base = [W.FLUID, W.STEEL, W.CEMENT, W.ROCK]
+    mats = [base[q % 4] for q in range(n_mat)]
+    cid = rng.integers(0, n_mat, size=g.shape).astype(np.uint16)
+    cid[:, 0, :] = 0
+    med = W.Medium(g, cid, *(np.array([m[q] for m in mats]) for q in range(3)))
+    steps = 8
+    sc = W.Scenario("march", med, W.Source(r=0.009, theta=2.0, z=0.012, f0=60e3), W.on_axis_receivers([0.0]), steps=steps)
+    sc.pml_on = pml_on
+    scale = 1.0 / (1000.0 * 1500.0) if storage.startswith("f16") else 1e-7
+    v0 = {n: (scale * rng.standard_normal(g.shape)).astype(np.float32) for n in ("vr", "vp", "vz")}
+    v0["vr"][:, 0] = 0
+    v0["vz"][:, :, -1] = 0
+    exact = tile != 2324 or storage != "f32" or not pml_on or n_mat > 2048
+    with Simulation(sc, kernel="split", tile=tile, storage=storage) as a, \
+            Simulation(sc, kernel="split", tile=2335, storage=storage) as b:
+        for n in v0:
+            a.set_field(n, v0[n])
+            b.set_field(n, v0[n])
+        a.step(steps)
+        b.step(steps)
+        for n in oracle.FIELDS:
+            x, y = a.field(n), b.field(n)
+            assert np.abs(y).max() > 0, n
+            assert np.abs(x - y).max() <= (0 if exact else 2e-5) * np.abs(y).max(), n
