@@ -238,7 +238,7 @@ def cpu_sample(sc, seconds=15.0, nz=128):
 
 def bench_batch(stream, n_cases=64, steps=60, warm=8, rank=0, ws=1, pg=None):
     """Batched scenarios (the 64 cement-hardening cases, uneven Nz) in one
-    persistent launch per kernel per step, against the same cases run one
+    batch (large cases in their own launches, small ones sharing them), against the same cases run one
     after another with the single-well path.  Throughput is reported in full
     6000-step scenarios per second, measured over `steps` steps.  Under
     torchrun the cases are sharded round robin over the ranks (weak in
@@ -369,7 +369,7 @@ def bench_refined(stream, sc, uniform_value, uniform_dt, steps=400, warm=20, til
             "gcell_updates_per_s": cells * steps / t / 1e9, "cells_per_step": cells,
             "uniform_cells_per_step": uniform_cells, "dt": dt, "uniform_dt": uniform_dt,
             "zones": [{"first_row": a, "rows": b, "nth": c} for a, b, c in zones], "steps_timed": steps,
-            "split_codes": tile or 22852324,
+            "split_codes": tile or 2324,
             "error": "GPU vs the refined FP64 oracle: fields <= 2e-5 of scale, traces <= 1e-4 rel-L2 (tested)"}
 
 
