@@ -8,10 +8,10 @@
 // than the bytes.  The march keeps 13 loads a thread in flight throughout, reads
 // the theta neighbours once (they are the present values of the plane before or
 // after), and with 32-bit offsets and the material table in shared memory takes
-// 410.  196 x 64 x 1056 cells, BF16: 217 us a step tile by tile, 193 here;
+// 420.  196 x 64 x 1056 cells, BF16: 217 us a step tile by tile, 193 here;
 // FP16-SR 342 and 285; FP32 on 136 x 32 x 3104 cells 294 and 269.  Its interior
-// launches reach 62 to 64 % of the DRAM throughput (47 to 53 % tile by tile); what
-// is left is issue slots (58 % busy) and the start of every run.
+// launches reach 66 and 57 % of the DRAM throughput (53 and 46 % tile by tile); what
+// is left is issue slots (57 to 61 % busy) and the start of every run.
 //
 // The radial layer (RAD) takes the same march in FP32 with its memory variables
 // loaded ahead too, two blocks an SM: 212 x 64 x 8224 cells, the launches beside
