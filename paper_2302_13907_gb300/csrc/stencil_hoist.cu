@@ -5,8 +5,9 @@
 // {rho}, {1/mu}, {lambda, lambda + 2 mu}.  Same thread layout (four z cells
 // per thread, 16-byte loads, block = 32 x 4 threads, theta fastest across
 // blocks), same arithmetic, same in-place update; variants with two z cells
-// per thread (8-byte loads, fewer registers), and interior / edge split
-// launches (a lean-only kernel on the interior tiles).
+// per thread (8-byte loads, fewer registers), interior / edge split launches
+// (a lean-only kernel on the interior tiles), the march along theta
+// (hoist_run.cuh) and one launch per half for batches and small grids.
 #include <algorithm>
 
 #include "hoist_run.cuh"

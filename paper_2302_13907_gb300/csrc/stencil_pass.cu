@@ -33,7 +33,7 @@
 //
 // Measured: 196 x 64 x 8224 cells 1.27 ms a launch (74 bytes a cell: 5.5 TB/s)
 // where the split halves take 0.83 + 1.03 ms on the same cells; the step with its
-// edge launches 1.74 ms against 2.15.  136 x 32 x 3104: 0.26 ms against 0.29.
+// edge launches 1.68 ms (1.73 before the radial layer was marched) against 2.15.  136 x 32 x 3104: 0.26 ms against 0.29.
 //
 // What bounds it: DRAM.  Halo rows and columns (11 x 128 read for 9 x 120
 // owned) are shared with blocks that run at the same time and come from L2.
