@@ -343,6 +343,20 @@ __device__ __forceinline__ float stretch_reg(float &psi, float a, float b, float
   return D + psi;
 }
 
+// a b + c d with the first product inside the fused multiply-add.  Where two
+// kernels compute the same cell, the sums of products are written out so, one way
+// round or the other, because the compiler's own choice differs between bodies;
+// with the choices it makes in the lean body all of them give that body's bits, in
+// 16-bit storage too, where a last bit of FP32 decides a rounding and 128 steps
+// spread it.
+__device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+
+// cell k of a row of the interior whose aligned pair of cells lies clear of the z
+// PML: the cells that a kernel with two cells per thread gives to the lean body
+__device__ __forceinline__ bool lean_pair(const KParams &p, int i, int k) {
+  return i < p.nr && (k & ~1) >= p.pml_z && (k & ~1) + 2 < p.NZ - p.pml_z;
+}
+
 template <int NV>
 __device__ __forceinline__ void zero(float (&d)[NV]) {
 #pragma unroll
@@ -372,9 +386,10 @@ __device__ __forceinline__ void zero_ids(int (&o)[NV]) {
 // lie inside NZ and outside the z PML (no z memory variable, no z bound
 // check); by default the same as LEAN.  LEAN: the NV cells are interior (no PML
 // memory variable, all inside NZ, k0 + NV < NZ); the kernels pick the lean
-// body per thread, or run it alone on the interior tiles.  out: the set written
-// (null: in place).
-template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN>
+// body per thread, or run it alone on the interior tiles.  PAIRS: the general
+// body gives the cells it shares with the lean one (lean_pair) the lean body's
+// bits.  out: the set written (null: in place).
+template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN, bool PAIRS = false>
 __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, const int i, const int k0,
                                                const OutSet *out = nullptr) {
   void *const *fo = out ? out->f : p.f;
@@ -493,47 +508,50 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
     const bool zp = zl && (k < pz || k >= NZ - pz);
     const int kz = k < pz ? k : k - (NZ - 2 * pz);
     const float4 abz = zp ? __ldg(p.ab_z + k) : z4();
+    const bool lean = PAIRS && lean_pair(p, i, k);
     const float srr_e = a_srr[e], spp_e = a_spp[e], srp_e = a_srp[e];
     const float srz_e = a_srz[e], spz_e = a_spz[e], szz_e = a_szz[e];
     const float srz_m1 = e ? a_srz[e - 1] : srz_km, spz_m1 = e ? a_spz[e - 1] : spz_km;
     // v_r at (r_i, theta_j, z_k), i >= 1
     if (im) {
-      float Dr = (srr_e - m_srr[e]) * idr;
-      float Q = (0.5f * (srr_e + m_srr[e]) - 0.5f * (spp_e + m_spp[e]) + (srp_e - jm_srp[e]) * idth) *
-                inv_ri;
-      float Dz = (srz_e - srz_m1) * idz;
+      const float dr = srr_e - m_srr[e], dz = srz_e - srz_m1;
+      const float q = 0.5f * (srr_e + m_srr[e]) - 0.5f * (spp_e + m_spp[e]) + (srp_e - jm_srp[e]) * idth;
+      float Dr = dr * idr, Q = q * inv_ri, Dz = dz * idz;
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vr[e], abr.x, abr.y, Dr) : stretch(p.psr[R_VR] + cr + e, abr.x, abr.y, Dr));
         Q = (PRE ? stretch_reg(uq_vr[e], abq.x, abq.y, Q) : stretch(p.psr[Q_VR] + cr + e, abq.x, abq.y, Q));
       }
       if (zp) Dz = (PRE ? stretch_reg(uz_vr[e], abz.x, abz.y, Dz) : stretch(p.psz[Z_VR] + czrow + kz, abz.x, abz.y, Dz));
-      out_r[e] += vel_coef(dtv, rho_m[e] + rho_c[e]) * (Dr + Q + Dz);
+      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_ri)) : Dr + Q + Dz;
+      out_r[e] += vel_coef(dtv, rho_m[e] + rho_c[e]) * t;
     }
     // v_phi at (r_{i+1/2}, theta_{j+1/2}, z_k)
     {
       const float s1 = p_srp[e];
-      float Dr = (s1 - srp_e) * idr;
-      float Q = ((s1 + srp_e) + (jp_spp[e] - spp_e) * idth) * inv_rh;
-      float Dz = (spz_e - spz_m1) * idz;
+      const float dr = s1 - srp_e, q = (s1 + srp_e) + (jp_spp[e] - spp_e) * idth, dz = spz_e - spz_m1;
+      float Dr = dr * idr, Q = q * inv_rh, Dz = dz * idz;
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vp[e], abr.z, abr.w, Dr) : stretch(p.psr[R_VP] + cr + e, abr.z, abr.w, Dr));
         Q = (PRE ? stretch_reg(uq_vp[e], abq.z, abq.w, Q) : stretch(p.psr[Q_VP] + cr + e, abq.z, abq.w, Q));
       }
       if (zp) Dz = (PRE ? stretch_reg(uz_vp[e], abz.x, abz.y, Dz) : stretch(p.psz[Z_VP] + czrow + kz, abz.x, abz.y, Dz));
-      out_p[e] += vel_coef(dtv, rho_c[e] + rho_j[e]) * (Dr + Q + Dz);
+      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_rh)) : Dr + Q + Dz;
+      out_p[e] += vel_coef(dtv, rho_c[e] + rho_j[e]) * t;
     }
     // v_z at (r_{i+1/2}, theta_j, z_{k+1/2}), k + 1 < NZ
     if (ZIN || k + 1 < NZ) {
       const float s1 = p_srz[e];
-      float Dr = (s1 - srz_e) * idr;
-      float Q = (0.5f * (s1 + srz_e) + (spz_e - jm_spz[e]) * idth) * inv_rh;
-      float Dz = ((e < NV - 1 ? a_szz[e + 1] : szz_k4) - szz_e) * idz;
+      const float dr = s1 - srz_e, dz = (e < NV - 1 ? a_szz[e + 1] : szz_k4) - szz_e;
+      const float q = lean ? mul_add2(0.5f, s1 + srz_e, spz_e - jm_spz[e], idth)
+                           : 0.5f * (s1 + srz_e) + (spz_e - jm_spz[e]) * idth;
+      float Dr = dr * idr, Q = q * inv_rh, Dz = dz * idz;
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vz[e], abr.z, abr.w, Dr) : stretch(p.psr[R_VZ] + cr + e, abr.z, abr.w, Dr));
         Q = (PRE ? stretch_reg(uq_vz[e], abq.z, abq.w, Q) : stretch(p.psr[Q_VZ] + cr + e, abq.z, abq.w, Q));
       }
       if (zp) Dz = (PRE ? stretch_reg(uz_vz[e], abz.z, abz.w, Dz) : stretch(p.psz[Z_VZ] + czrow + kz, abz.z, abz.w, Dz));
-      out_z[e] += vel_coef(dtv, rho_c[e] + rho_c[e + 1]) * (Dr + Q + Dz);
+      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_rh)) : Dr + Q + Dz;
+      out_z[e] += vel_coef(dtv, rho_c[e] + rho_c[e + 1]) * t;
     }
   }
   const SrKey sk = body_key<T>(p, j, i, k0);
@@ -567,7 +585,7 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
 // in which other blocks wrote them, and the cell's own stresses are read and
 // written streaming (last use in the launch).  out: the set that holds the new
 // velocities and is written (null: in place).
-template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN, bool CG = false>
+template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN, bool CG = false, bool PAIRS = false>
 __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, const int i, const int k0,
                                                const OutSet *out = nullptr) {
   void *const *fo = out ? out->f : p.f;
@@ -708,6 +726,7 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
     const bool zp = zl && (k < pz || k >= NZ - pz);
     const int kz = k < pz ? k : k - (NZ - 2 * pz);
     const float4 abz = zp ? __ldg(p.ab_z + k) : z4();
+    const bool lean = PAIRS && lean_pair(p, i, k);
     const float vr_e = a_vr[e], vp_e = a_vp[e], vz_e = a_vz[e];
     const float vr_e1 = e < NV - 1 ? a_vr[e + 1] : vr_k4, vp_e1 = e < NV - 1 ? a_vp[e + 1] : vp_k4;
     const float vz_m1 = e ? a_vz[e - 1] : vz_km;
@@ -723,40 +742,50 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
       }
       if (zp) ezz = (PRE ? stretch_reg(uz_zz[e], abz.x, abz.y, ezz) : stretch(p.psz[Z_EZZ] + czrow + kz, abz.x, abz.y, ezz));
       const float l = lam[e].x, l2m = lam[e].y;
-      orr[e] += dts * (l2m * err + l * (epp + ezz)) + src[e];
-      opp[e] += dts * (l2m * epp + l * (err + ezz)) + src[e];
-      ozz[e] += dts * (l2m * ezz + l * (err + epp)) + src[e];
+      if (lean) {
+        epp = __fmul_rn(mul_add2(0.5f, vr_e + vr1, vp_e - jm_vp[e], idth), inv_rh);
+        orr[e] = __fadd_rn(orr[e], __fmaf_rn(dts, mul_add2(l2m, err, l, __fadd_rn(epp, ezz)), src[e]));
+        opp[e] = __fadd_rn(opp[e], __fmaf_rn(dts, mul_add2(l, __fadd_rn(err, ezz), l2m, epp), src[e]));
+        ozz[e] = __fadd_rn(ozz[e], __fmaf_rn(dts, mul_add2(l2m, ezz, l, __fadd_rn(err, epp)), src[e]));
+      } else {
+        orr[e] += dts * (l2m * err + l * (epp + ezz)) + src[e];
+        opp[e] += dts * (l2m * epp + l * (err + ezz)) + src[e];
+        ozz[e] += dts * (l2m * ezz + l * (err + epp)) + src[e];
+      }
     }
     if (im) {
       // s_rphi at (r_i, theta_{j+1/2}, z_k)
       {
-        float gr = (vp_e - m_vp[e]) * idr;
-        float Q = ((jp_vr[e] - vr_e) * idth - 0.5f * (vp_e + m_vp[e])) * inv_ri;
+        const float dr = vp_e - m_vp[e];
+        const float q = lean ? mul_add2(jp_vr[e] - vr_e, idth, -0.5f, vp_e + m_vp[e])
+                             : (jp_vr[e] - vr_e) * idth - 0.5f * (vp_e + m_vp[e]);
+        float gr = dr * idr, Q = q * inv_ri;
         if (rp) {
           gr = (PRE ? stretch_reg(ur_rp[e], abr.x, abr.y, gr) : stretch(p.psr[R_GRP] + cr + e, abr.x, abr.y, gr));
           Q = (PRE ? stretch_reg(uq_rp[e], abq.x, abq.y, Q) : stretch(p.psr[Q_GRP] + cr + e, abq.x, abq.y, Q));
         }
         const float mu = mu_harm(imu_m[e] + imu_c[e] + imu_jm[e] + imu_j[e]);
-        orp[e] += dts * mu * (gr + Q);
+        orp[e] += dts * mu * (lean ? mul_add2(dr, idr, q, inv_ri) : gr + Q);
       }
       // s_rz at (r_i, theta_j, z_{k+1/2})
       if (ZIN || k + 1 < NZ) {
-        float gz = (vr_e1 - vr_e) * idz;
-        float gr = (vz_e - m_vz[e]) * idr;
+        const float dz = vr_e1 - vr_e, dr = vz_e - m_vz[e];
+        float gz = dz * idz, gr = dr * idr;
         if (zp) gz = (PRE ? stretch_reg(uz_rz[e], abz.z, abz.w, gz) : stretch(p.psz[Z_GRZ] + czrow + kz, abz.z, abz.w, gz));
         if (rp) gr = (PRE ? stretch_reg(ur_rz[e], abr.x, abr.y, gr) : stretch(p.psr[R_GRZ] + cr + e, abr.x, abr.y, gr));
         const float mu = mu_harm(imu_m[e] + imu_c[e] + imu_m[e + 1] + imu_c[e + 1]);
-        orz[e] += dts * mu * (gz + gr);
+        orz[e] += dts * mu * (lean ? mul_add2(dz, idz, dr, idr) : gz + gr);
       }
     }
     // s_phiz at (r_{i+1/2}, theta_{j+1/2}, z_{k+1/2})
     if (ZIN || k + 1 < NZ) {
+      const float dz = vp_e1 - vp_e;
       float Q = (jp_vz[e] - vz_e) * idth * inv_rh;
-      float gz = (vp_e1 - vp_e) * idz;
+      float gz = dz * idz;
       if (rp) Q = (PRE ? stretch_reg(uq_pz[e], abq.z, abq.w, Q) : stretch(p.psr[Q_GPZ] + cr + e, abq.z, abq.w, Q));
       if (zp) gz = (PRE ? stretch_reg(uz_pz[e], abz.z, abz.w, gz) : stretch(p.psz[Z_GPZ] + czrow + kz, abz.z, abz.w, gz));
       const float mu = mu_harm(imu_c[e] + imu_j[e] + imu_c[e + 1] + imu_j[e + 1]);
-      opz[e] += dts * mu * (Q + gz);
+      opz[e] += dts * mu * (lean ? __fmaf_rn(dz, idz, __fmul_rn(__fmul_rn(jp_vz[e] - vz_e, idth), inv_rh)) : Q + gz);
     }
   }
   const SrKey sk = body_key<T>(p, j, i, k0);

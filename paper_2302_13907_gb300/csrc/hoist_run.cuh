@@ -43,13 +43,6 @@ __device__ __forceinline__ unsigned ld_ahead2(const void *p) {
   return v;
 }
 
-// a b + c d with the first product inside the fused multiply-add.  The sums of
-// products below are written out so, one way round or the other, because the
-// compiler's own choice differs between this loop and the tile kernels; with the
-// choices it makes there the march gives their bits, in 16-bit storage too,
-// where a last bit of FP32 decides a rounding and 128 steps spread it.
-__device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
-
 // four values of a row, and one, as stored
 template <typename T>
 struct Raw4 {

@@ -143,10 +143,13 @@ __device__ __forceinline__ void radial_cells_step(const KParams &p, int j, int i
   if (VEL) vel_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
   else str_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
 }
+// The z ends also hold cells beside the layer that no memory variable touches (up
+// to three of a cut group, up to a quarter of a tile): PAIRS gives them the bits of
+// the lean body, so that where the cut lies does not show in the fields.
 template <typename T, int NV, bool VEL>
 __device__ __forceinline__ void end_cells_step(const KParams &p, int j, int i, int k0, const OutSet *out = nullptr) {
-  if (VEL) vel_hoist_body<T, NV, false, true>(p, j, i, k0, out);
-  else str_hoist_body<T, NV, false, true>(p, j, i, k0, out);
+  if (VEL) vel_hoist_body<T, NV, false, true, false, true>(p, j, i, k0, out);
+  else str_hoist_body<T, NV, false, true, false, false, true>(p, j, i, k0, out);
 }
 
 template <typename T, int NV, int MINB, bool VEL>

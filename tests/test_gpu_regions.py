@@ -88,3 +88,39 @@ def test_march_along_theta(tile, storage, nth, nr, pml_r, nz, pml_z, pml_on, n_m
             x, y = a.field(n), b.field(n)
             assert np.abs(y).max() > 0, n
             assert np.abs(x - y).max() <= (0 if exact else 2e-5) * np.abs(y).max(), n
+
+
+@pytest.mark.parametrize("tile", [2204, 2216, 2224, 2256, 2275, 2285, 2304, 2314, 2324])
+@pytest.mark.parametrize("storage,steps", [("f32", 3), ("bf16", 40), ("f16", 40)])
+@pytest.mark.parametrize("nz,pml_z", [
+    (146, 3),   # the z ends hold a sliver of lean groups and an odd pair at either side
+    (60, 98),   # the same below the lean cells
+    (117, 2),   # lean cells up to one pair from the layer
+    (252, 4),   # cuts on the layer's first cell
+])
+def test_no_trace_of_the_cut_in_the_fields(tile, storage, steps, nz, pml_z):
+    """Where a split code cuts a row into lean cells and z ends does not show:
+    every field has the bits of the kernel that decides per pair of cells (2106).
+    (No radial layer: its body has its own order of sums.)"""
+    from paper_2302_13907_gb300.binding import Simulation
+    g = W.Grid(nr=9, nth=6, nz=nz, pml_r=0, pml_z=pml_z, dr=0.004, dz=0.003)
+    rng = np.random.default_rng(nz)
+    mats = [W.FLUID, W.STEEL, W.CEMENT, W.ROCK]
+    cid = rng.integers(0, len(mats), size=g.shape).astype(np.uint16)
+    cid[:, 0, :] = 0
+    med = W.Medium(g, cid, *(np.array([m[q] for m in mats]) for q in range(3)))
+    sc = W.Scenario("cut", med, W.Source(r=0.009, theta=2.0, z=0.012, f0=60e3), W.on_axis_receivers([0.0]), steps=steps)
+    v = {n: rng.standard_normal(g.shape).astype(np.float32) / (1000 * 1500) for n in ("vr", "vp", "vz")}
+    v["vr"][:, 0] = 0
+    v["vz"][:, :, -1] = 0
+    with Simulation(sc, kernel="split", tile=tile, storage=storage) as a, \
+            Simulation(sc, kernel="split", tile=2106, storage=storage) as b:
+        for n in v:
+            a.set_field(n, v[n])
+            b.set_field(n, v[n])
+        a.step(steps)
+        b.step(steps)
+        for n in oracle.FIELDS:
+            x, y = a.field(n), b.field(n)
+            assert np.abs(y).max() > 0, n
+            assert np.array_equal(x, y), (n, np.flatnonzero((x != y).any((0, 1))))
