@@ -6,10 +6,10 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <map>
 #include <mutex>
 #include <string>
-#include <tuple>
 #include <vector>
 
 #include "sim_state.cuh"
@@ -271,9 +271,10 @@ static int build_pass_maps(sim_t *h) {
 }
 
 // Autotuner: time each tile height on the still-zero state with the source
-// disabled (the state stays zero), keep the fastest; cached per grid shape.
+// disabled (the state stays zero), keep the fastest; cached per grid shape and
+// all that decides which codes a handle can run.
 static std::mutex g_tune_mu;
-static std::map<std::tuple<int, int, int, int, int, int>, std::pair<int, int>> g_tune;  // pick, best split code
+static std::map<std::array<int, 8>, std::pair<int, int>> g_tune;  // pick, best split code
 
 static cudaError_t launch_fused_any(int storage, int code, const FusedMaps &maps, const FusedParams &fp,
                                     cudaStream_t s) {
@@ -367,10 +368,15 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
   const bool allow_split = kernel == SIM_KERNEL_AUTO || kernel == SIM_KERNEL_SPLIT;
   int dev = h->device, maxsm = 0;
   cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // point forces rule out the sweep kernel: they key a separate choice
+  // the one-pass step needs the second set, room for the material table beside
+  // its staged planes, and enough lean cells
+  int r1, z0, z1;
+  const bool pass_ok = kernel == SIM_KERNEL_AUTO && h->two_sets && h->storage == SIM_STORAGE_F32 &&
+                       pass_smem_bytes(h->n_mat) <= (size_t)maxsm && pass_region(h->kp, &r1, &z0, &z1);
+  // point forces rule out the sweep kernel, a slab all but the interior / edge codes
   const bool force = h->src_kind == 1 || h->src_kind == 2;
-  auto key = std::make_tuple(dev, h->grid.nth, h->NR, h->NZ, h->stencil_storage * 8 + kernel,
-                             (h->kp.pml_r > 0 ? 1 : 0) + (force ? 2 : 0) + (h->two_sets ? 4 : 0));
+  const std::array<int, 8> key = {dev, h->grid.nth, h->NR, h->NZ, h->kp.nr, h->kp.pml_z, h->stencil_storage * 8 + kernel,
+                                  (force ? 1 : 0) + (h->fused ? 2 : 0) + (h->slab ? 4 : 0) + (pass_ok ? 8 : 0)};
   if (!forced) {
     std::lock_guard<std::mutex> g(g_tune_mu);
     auto it = g_tune.find(key);
@@ -398,9 +404,6 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
     if (v && c) pick = forced;
   }
   h->split_rt = 2224;  // half steps beside a forced one-pass code
-  int r1, z0, z1;
-  const bool pass_ok = kernel == SIM_KERNEL_AUTO && h->two_sets && h->storage == SIM_STORAGE_F32 &&
-                       pass_smem_bytes(h->n_mat) <= (size_t)maxsm && pass_region(h->kp, &r1, &z0, &z1);
   if (pass_ok && (!forced || is_pass(forced))) {
     int rc = build_pass_maps(h);
     if (rc) return rc;

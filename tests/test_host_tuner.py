@@ -1,0 +1,54 @@
+"""The kernel choice of AUTO and the memory it keeps, on the CPU against a
+stand-in for the CUDA runtime (fake_runtime.py): kernels cost what the test says."""
+import pytest
+
+from fake_runtime import run
+
+WELLS = """
+for k, us in ((b"fused", 100.0), (b"march", 100.0), (b"sweep", 100.0), (b"hoist", 10.0), (b"split", 10.0),
+              (b"hoist_edge", 0.1), (b"hoist_rim", 0.1)):
+    fake.fake_cost(k, us)
+
+def well(nr=24, nth=8, nz=80, pml_r=4, pml_z=4, n_mat=4, kind=0, receivers=1):
+    g = W.Grid(nr=nr, nth=nth, nz=nz, pml_r=pml_r, pml_z=pml_z, dr=0.004, dz=0.003)
+    mats = [(W.FLUID, W.ROCK)[min(q, 1)] for q in range(n_mat)]
+    cid = np.ones(g.shape, np.uint16)
+    cid[:, 0, :] = 0
+    med = W.Medium(g, cid, *(np.array([m[q] for m in mats]) for q in range(3)))
+    rec = W.on_axis_receivers([0.0] * receivers)
+    return W.Scenario("t", med, W.Source(z=0.03, f0=60e3, kind=kind), rec, steps=4)
+
+def step(sc, **kw):
+    with B.Simulation(sc, **kw) as s:
+        try:
+            s.step(4)
+            ok = ""
+        except B.SimError as e:
+            ok = str(e)
+        return [s.config()[0], ok]
+"""
+
+
+@pytest.mark.parametrize("other", [
+    "n_mat=2197",              # a table that leaves no room beside the staged planes
+    "nz=20, pml_z=34",         # the same stored cells, 16 of a row lean
+    "nr=4, pml_r=24",          # the same rows, three lean
+])
+def test_a_cached_one_pass_choice_goes_to_wells_that_can_run_it_only(other):
+    """The tuner's cache hands a well the choice of an earlier one only where all
+    that decides whether the choice runs is the same, in either order."""
+    r = run(WELLS + f"""
+fake.fake_cost(b"pass_step", 0.01)
+out["first"] = step(well())
+out["other"] = step(well({other}))
+out["again"] = step(well())
+out["forced"] = step(well(), tile=4001)
+""")
+    assert r["first"] == [6, ""] and r["again"] == [6, ""] and r["forced"] == [6, ""], r
+    assert r["other"][1] == "" and r["other"][0] != 6, r
+    r = run(WELLS + f"""
+fake.fake_cost(b"pass_step", 0.01)
+out["other"] = step(well({other}))
+out["first"] = step(well())
+""")
+    assert r["first"] == [6, ""] and r["other"][1] == "" and r["other"][0] != 6, r
