@@ -36,6 +36,15 @@ static int dev_alloc(sim_t *h, void **p, size_t bytes) {
   return SIM_OK;
 }
 
+// gives back what dev_alloc took for the last n arrays (of `bytes` in all)
+static void dev_free_last(sim_t *h, size_t n, size_t bytes) {
+  for (; n > 0 && !h->allocs.empty(); n--) {
+    cudaFree(h->allocs.back());
+    h->allocs.pop_back();
+  }
+  h->bytes -= bytes;
+}
+
 // Ricker pulse, dominant frequency f0, delay 2/f0 (Sec. 2 of the paper)
 double cwell::ricker(double t, double f0) {
   double a = M_PI * f0 * (t - 2.0 / f0);
@@ -363,16 +372,20 @@ static cudaError_t time_graph(sim_t *h, cudaEvent_t a, cudaEvent_t b, float *ms,
   return e;
 }
 
+// what the one-pass step needs beside a second set: FP32, room for the material
+// table beside its staged planes, and enough lean cells
+static bool pass_fits(const sim_t *h) {
+  int maxsm = 0, r1, z0, z1;
+  cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+  return h->storage == SIM_STORAGE_F32 && pass_smem_bytes(h->n_mat) <= (size_t)maxsm && pass_region(h->kp, &r1, &z0, &z1);
+}
+
 static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
   SideScope side_scope(h);
   const bool allow_split = kernel == SIM_KERNEL_AUTO || kernel == SIM_KERNEL_SPLIT;
   int dev = h->device, maxsm = 0;
   cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // the one-pass step needs the second set, room for the material table beside
-  // its staged planes, and enough lean cells
-  int r1, z0, z1;
-  const bool pass_ok = kernel == SIM_KERNEL_AUTO && h->two_sets && h->storage == SIM_STORAGE_F32 &&
-                       pass_smem_bytes(h->n_mat) <= (size_t)maxsm && pass_region(h->kp, &r1, &z0, &z1);
+  const bool pass_ok = kernel == SIM_KERNEL_AUTO && h->two_sets && pass_fits(h);
   // point forces rule out the sweep kernel, a slab all but the interior / edge codes
   const bool force = h->src_kind == 1 || h->src_kind == 2;
   const std::array<int, 8> key = {dev, h->grid.nth, h->NR, h->NZ, h->kp.nr, h->kp.pml_z, h->stencil_storage * 8 + kernel,
@@ -819,20 +832,6 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
         if ((rc = dev_alloc(h, (void **)&h->psz2[q], h->psz_elems * 4))) return bail(rc);
     }
   }
-  h->two_sets = h->fused;
-  if (opts->kernel == SIM_KERNEL_AUTO && !h->fused && !slab && opts->storage == SIM_STORAGE_F32 && source->kind != 0) {
-    // the point forces and the torsion ring rule out the fused kernels but not
-    // the one-pass step: it gets its second set where that takes no more than a
-    // third of the free memory and stays under the cap
-    const size_t set = NF * ((fbytes + 255) & ~size_t(255));
-    size_t free_b = 0, total_b = 0;
-    if ((e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bail(cuda_fail(h, e, "cudaMemGetInfo"));
-    if (3 * set <= free_b && (!h->mem_cap || h->bytes + 2 * set <= h->mem_cap)) {
-      for (int q = 0; q < NF; q++)
-        if ((rc = dev_alloc(h, &h->f2[q], fbytes))) return bail(rc);
-      h->two_sets = true;
-    }
-  }
   if ((rc = dev_alloc(h, (void **)&h->id, (size_t)nth * NR * NZp * 2))) return bail(rc);
   if ((rc = dev_alloc(h, (void **)&h->mat, mat.size() * sizeof(float4)))) return bail(rc);
   if ((rc = dev_alloc(h, (void **)&h->m_rho, mat.size() * 4))) return bail(rc);
@@ -935,21 +934,6 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
   h->ip.n_wav = h->n_wav;
   h->ip.step = h->step;
   for (int q = 0; q < NF; q++) h->ip.f[q] = h->f[q];
-  std::vector<float> fw;  // point force: weight of each azimuthal node
-  float *d_fw = nullptr;
-  int force_i = -1;
-  if ((source->kind == 1 || source->kind == 2) && !ifld.empty() && h->two_sets) {
-    fw.assign(nth, 0.f);
-    for (size_t q = 0; q < ioff.size(); q++) {
-      const int j = (int)(ioff[q] / p.plane);
-      force_i = (int)(ioff[q] % p.plane / NZp);
-      fw[j] = iw[q];
-    }
-    if ((rc = dev_alloc(h, (void **)&d_fw, nth * 4))) return bail(rc);
-    if ((e = cudaMemcpyAsync(d_fw, fw.data(), nth * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-      return bail(cuda_fail(h, e, "upload force"));
-  }
   RParams &r = h->rp;
   r.nth = nth;
   r.NR = NR;
@@ -965,30 +949,6 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
   r.traces = h->traces;
   r.step = h->step;
   r.status = h->status;
-  if (h->two_sets)
-    for (int par = 0; par < 2; par++) {  // step from set par to the other
-      PassParams &q = h->pp[par];
-      void **cur = par == 0 ? h->f : h->f2, **nxt = par == 0 ? h->f2 : h->f;
-      q.k = p;
-      h->ip2[par] = h->ip;
-      for (int k = 0; k < NF; k++) {
-        q.k.f[k] = cur[k];
-        q.out.f[k] = h->ip2[par].f[k] = nxt[k];
-      }
-      q.status = h->status;
-      q.n_mat = h->n_mat;
-      q.force_i = force_i;
-      q.force_k = (int)ks - l0;
-      q.force_vz = source->kind == 2;
-      q.force_w = d_fw;
-      q.force_wav = d_iwav;
-      h->rp2[par] = r;
-      h->rp2[par].srr = nxt[F_SRR];
-      h->rp2[par].spp = nxt[F_SPP];
-      h->rp2[par].szz = nxt[F_SZZ];
-      int r1, z0, z1;
-      h->force_outside = force_i >= 0 && !(pass_region(q.k, &r1, &z0, &z1) && force_i < r1 && q.force_k >= z0 && q.force_k < z1);
-    }
   if (opts->watchdog_every > 0) {
     h->watch_every = opts->watchdog_every;
     if ((rc = dev_alloc(h, (void **)&h->watch_acc, 4 * sizeof(double)))) return bail(rc);
@@ -1018,6 +978,65 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
       w.acc = h->watch_acc;
     }
   }
+  h->two_sets = h->fused;
+  // The point forces and the torsion ring rule out the fused kernels but not the
+  // one-pass step.  Its second set comes after everything the handle cannot do
+  // without, where the step can run and the tuner may pick it, if the set takes no
+  // more than a third of the free memory and stays under the cap; a handle that
+  // cannot have it is created without.  Given back below unless the step is picked.
+  const size_t before = h->bytes, arrays = h->allocs.size();
+  std::vector<float> fw;  // point force: weight of each azimuthal node
+  float *d_fw = nullptr;
+  int force_i = -1;
+  if (opts->kernel == SIM_KERNEL_AUTO && !h->fused && !slab && source->kind != 0 && (!opts->tile || is_pass(opts->tile)) &&
+      pass_fits(h)) {
+    const size_t set = NF * ((fbytes + 255) & ~size_t(255));
+    size_t free_b = 0, total_b = 0;
+    if ((e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return bail(cuda_fail(h, e, "cudaMemGetInfo"));
+    rc = 3 * set <= free_b ? SIM_OK : SIM_ENOMEM;
+    for (int q = 0; q < NF && !rc; q++) rc = dev_alloc(h, &h->f2[q], fbytes);
+    if (!rc && source->kind != 3) {
+      fw.assign(nth, 0.f);
+      for (size_t q = 0; q < ioff.size(); q++) {
+        const int j = (int)(ioff[q] / p.plane);
+        force_i = (int)(ioff[q] % p.plane / NZp);
+        fw[j] = iw[q];
+      }
+      rc = dev_alloc(h, (void **)&d_fw, nth * 4);
+      if (!rc && ((e = cudaMemcpyAsync(d_fw, fw.data(), nth * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+                  (e = cudaStreamSynchronize(st)) != cudaSuccess))
+        return bail(cuda_fail(h, e, "upload force"));
+    }
+    h->two_sets = rc == SIM_OK;
+    if (!h->two_sets) {
+      dev_free_last(h, h->allocs.size() - arrays, h->bytes - before);
+      h->err.clear();
+    }
+  }
+  if (h->two_sets)
+    for (int par = 0; par < 2; par++) {  // step from set par to the other
+      PassParams &q = h->pp[par];
+      void **cur = par == 0 ? h->f : h->f2, **nxt = par == 0 ? h->f2 : h->f;
+      q.k = p;
+      h->ip2[par] = h->ip;
+      for (int k = 0; k < NF; k++) {
+        q.k.f[k] = cur[k];
+        q.out.f[k] = h->ip2[par].f[k] = nxt[k];
+      }
+      q.status = h->status;
+      q.n_mat = h->n_mat;
+      q.force_i = force_i;
+      q.force_k = (int)ks - l0;
+      q.force_vz = source->kind == 2;
+      q.force_w = d_fw;
+      q.force_wav = d_iwav;
+      h->rp2[par] = r;
+      h->rp2[par].srr = nxt[F_SRR];
+      h->rp2[par].spp = nxt[F_SPP];
+      h->rp2[par].szz = nxt[F_SZZ];
+      int r1, z0, z1;
+      h->force_outside = force_i >= 0 && !(pass_region(q.k, &r1, &z0, &z1) && force_i < r1 && q.force_k >= z0 && q.force_k < z1);
+    }
   if (h->fused) {
     for (int par = 0; par < 2; par++) {
       FusedParams &f = h->fp[par];
@@ -1062,6 +1081,10 @@ static int create_impl(const sim_grid_t *grid, const sim_medium_t *medium, const
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return bail(cuda_fail(h, e, "autotune"));
     h->pass = is_pass(h->tile_rt);
+    if (h->two_sets && !h->pass) {
+      dev_free_last(h, h->allocs.size() - arrays, h->bytes - before);
+      h->two_sets = false;
+    }
     h->kernel = is_march(h->tile_rt) ? SIM_KERNEL_MARCH : is_sweep(h->tile_rt) ? SIM_KERNEL_SWEEP : SIM_KERNEL_SPLIT;
   }
   h->sweep = h->kernel == SIM_KERNEL_SWEEP;

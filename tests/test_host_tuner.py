@@ -52,3 +52,63 @@ out["other"] = step(well({other}))
 out["first"] = step(well())
 """)
     assert r["first"] == [6, ""] and r["other"][1] == "" and r["other"][0] != 6, r
+
+
+@pytest.mark.parametrize("kind", [1, 2, 3])
+def test_the_second_field_set_is_held_by_the_one_pass_step_only(kind):
+    """A point force or the torsion ring under AUTO: the second set is there while
+    the one-pass step runs, and neither with a split code asked for or picked nor
+    where the step cannot run."""
+    r = run(WELLS + f"""
+def size(sc, **kw):
+    with B.Simulation(sc, **kw) as s:
+        return [s.config()[0], s.device_bytes, fake.fake_used()]
+sc = lambda **kw: well(kind={kind}, **kw)
+if {kind} == 3:  # the ring lies in the rock
+    def sc(**kw):
+        x = well(kind=3, **kw)
+        x.source.r = 0.02
+        return x
+base = fake.fake_used()
+out["one set"] = size(sc(), kernel="split")
+out["tile"] = size(sc(), tile=2224)
+out["no room"] = size(sc(n_mat=2197))
+out["no room, split"] = size(sc(n_mat=2197), kernel="split")
+fake.fake_cost(b"pass_step", 0.01)
+out["picked"] = size(sc())
+fake.fake_cost(b"pass_step", 1000.0)
+out["not picked"] = size(sc(nz=81))
+out["not picked, split"] = size(sc(nz=81), kernel="split")
+fake.fake_cost(b"pass_step", 0.01)
+fake.fake_total(base + 3 * out["one set"][1])
+out["little memory"] = size(sc(nz=82))
+out["left"] = fake.fake_used() - base
+""")
+    assert r["tile"] == r["one set"]
+    assert r["no room"] == r["no room, split"]
+    assert r["picked"][0] == 6 and r["picked"][1] > 1.3 * r["one set"][1]
+    assert r["not picked"] == r["not picked, split"]
+    assert r["little memory"][0] == 1 and r["left"] == 0
+
+
+def test_a_memory_cap_that_held_one_set_still_does():
+    """A cap just above what one set of fields, the layers and the traces take:
+    the well is created without the second set."""
+    r = run(WELLS + """
+sc = well(kind=1, receivers=8)
+with B.Simulation(sc, kernel="split", max_steps=65536) as s:
+    out["bytes"] = s.device_bytes
+fake.fake_cost(b"pass_step", 0.01)
+with B.Simulation(sc, max_steps=65536, mem_cap=out["bytes"]) as s:
+    out["capped"] = [s.config()[0], s.device_bytes]
+    s.step(4)
+with B.Simulation(sc, max_steps=65536) as s:
+    out["free"] = s.config()[0]
+    set_bytes = s.device_bytes - out["bytes"]
+with B.Simulation(sc, max_steps=65536, mem_cap=out["bytes"] + set_bytes) as s:
+    out["room"] = s.config()[0]
+with B.Simulation(sc, max_steps=65536, mem_cap=out["bytes"] + set_bytes - 256) as s:
+    out["short"] = [s.config()[0], s.device_bytes]
+""")
+    assert r["capped"] == [1, r["bytes"]] and r["short"] == [1, r["bytes"]]
+    assert r["free"] == 6 and r["room"] == 6
