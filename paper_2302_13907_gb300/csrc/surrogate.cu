@@ -757,9 +757,20 @@ static cudaError_t forward(sur_t *s, int n) {
   return cudaGetLastError();
 }
 
-// Gradient into s->g and the loss kernel's LOSS_PARTS partial sums into lossp
-// (device), for the targets in s->tb; the handle's stream ends behind all of it.
-static cudaError_t backward(sur_t *s, int n, float *lossp) {
+// the handle's stream waits for what the side streams hold (the host does where
+// that cannot be enqueued)
+static cudaError_t join_sides(sur_t *s) {
+  cudaError_t first = cudaSuccess;
+  for (int k = 0; k < sur_t::SIDES; k++) {
+    cudaError_t e = cudaEventRecord(s->done[k], s->side[k]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s->stream, s->done[k], 0);
+    if (e != cudaSuccess) cudaStreamSynchronize(s->side[k]);
+    if (first == cudaSuccess) first = e;
+  }
+  return first;
+}
+
+static cudaError_t enqueue_backward(sur_t *s, int n, float *lossp) {
   const sur_cfg_t &c = s->cfg;
   cudaStream_t st = s->stream;
   cudaError_t e = cudaSuccess;
@@ -808,11 +819,16 @@ static cudaError_t backward(sur_t *s, int n, float *lossp) {
       return e;
     if (l > 0 && data(n, dims[l], dims[l + 1], s->gz16[l + 1], W16(s, 2 * l)) != cudaSuccess) return e;
   }
-  for (int k = 0; k < sur_t::SIDES; k++) {
-    if ((e = cudaEventRecord(s->done[k], s->side[k])) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(st, s->done[k], 0)) != cudaSuccess) return e;
-  }
   return cudaGetLastError();
+}
+
+// Gradient into s->g and the loss kernel's LOSS_PARTS partial sums into lossp
+// (device), for the targets in s->tb.  The handle's stream ends behind all of it,
+// also after a failure: what was enqueued by then still writes s->g and reads the
+// activations the next call overwrites.
+static cudaError_t backward(sur_t *s, int n, float *lossp) {
+  const cudaError_t e = enqueue_backward(s, n, lossp), j = join_sides(s);
+  return e != cudaSuccess ? e : j;
 }
 
 // the loss from the partial sums of a minibatch of n samples
