@@ -498,6 +498,7 @@ using namespace cwell;
 
 constexpr int COLSUM_PARTS = 4096;  // at most this many row chunks per column sum
 constexpr int LOSS_PARTS = 1024;    // blocks of the loss kernel
+constexpr int LOSS_KEEP = 1024;     // minibatches whose loss partials training keeps on the device (4 MB)
 
 struct sur_s {
   sur_cfg_t cfg{};
@@ -959,14 +960,16 @@ extern "C" int sur_train(sur_t *s, const float *X, const float *Y, int n, int ep
   const int Lf = L_out(s);
   const long long xrow = c.in_dim, yrow = (long long)Lf * c.out_ch;
   const int per_epoch = (n + batch - 1) / batch;
-  // the data, the epoch's order and every minibatch's loss partials stay on
-  // the device, so that no minibatch waits for the host; the losses are read
-  // once per epoch
+  // the data, the epoch's order and the loss partials of up to LOSS_KEEP
+  // minibatches stay on the device, so that no minibatch waits for the host: the
+  // losses are read once per epoch, or every LOSS_KEEP minibatches of a longer
+  // one (small batches of small cases must not take more memory than their data)
   float *dX = nullptr, *dY = nullptr, *dL = nullptr;
   int *dI = nullptr;
   cudaError_t e = cudaMalloc(&dX, (size_t)n * xrow * 4);
   if (e == cudaSuccess) e = cudaMalloc(&dY, (size_t)n * yrow * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&dL, (size_t)per_epoch * LOSS_PARTS * 4);
+  const int keep = std::min(per_epoch, LOSS_KEEP);
+  if (e == cudaSuccess) e = cudaMalloc(&dL, (size_t)keep * LOSS_PARTS * 4);
   if (e == cudaSuccess) e = cudaMalloc(&dI, (size_t)n * 4);
   if (e != cudaSuccess) {
     cudaFree(dX);
@@ -974,7 +977,7 @@ extern "C" int sur_train(sur_t *s, const float *X, const float *Y, int n, int ep
     cudaFree(dL);
     return sfail(s, SIM_ENOMEM, cudaGetErrorString(e));
   }
-  std::vector<float> lp((size_t)per_epoch * LOSS_PARTS);
+  std::vector<float> lp((size_t)keep * LOSS_PARTS);
   e = cudaMemcpyAsync(dX, X, (size_t)n * xrow * 4, cudaMemcpyHostToDevice, s->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dY, Y, (size_t)n * yrow * 4, cudaMemcpyHostToDevice, s->stream);
   std::vector<int> perm(n);
@@ -992,12 +995,22 @@ extern "C" int sur_train(sur_t *s, const float *X, const float *Y, int n, int ep
   for (int ep = 0; ep < epochs && e == cudaSuccess; ep++) {
     for (int q = n - 1; q > 0; q--) std::swap(perm[q], perm[rnd() % (uint64_t)(q + 1)]);
     if ((e = cudaMemcpyAsync(dI, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess) break;
+    double lsum = 0;
+    int read = 0;  // minibatches whose losses are in lsum
+    // the wait also keeps the host's order from being reshuffled before it is uploaded
+    auto read_losses = [&](int upto) {
+      e = cudaMemcpyAsync(lp.data(), dL, (size_t)(upto - read) * LOSS_PARTS * 4, cudaMemcpyDeviceToHost, s->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+      for (int q = read; q < upto && e == cudaSuccess; q++)
+        lsum += loss_of(s, lp.data() + (size_t)(q - read) * LOSS_PARTS, std::min(batch, n - q * batch));
+      read = upto;
+    };
     for (int b0 = 0; b0 < n && e == cudaSuccess; b0 += batch) {
       const int nb = std::min(batch, n - b0);
       k_gather<<<egrid(nb * xrow), 256, 0, s->stream>>>(dX, dI + b0, nb, xrow, s->xb);
       k_gather<<<egrid(nb * yrow), 256, 0, s->stream>>>(dY, dI + b0, nb, yrow, s->tb);
       if ((e = forward(s, nb)) != cudaSuccess) break;
-      if ((e = backward(s, nb, dL + (size_t)(b0 / batch) * LOSS_PARTS)) != cudaSuccess) break;
+      if ((e = backward(s, nb, dL + (size_t)(b0 / batch - read) * LOSS_PARTS)) != cudaSuccess) break;
       // cosine learning-rate schedule over all steps
       const float lr_t = 0.5f * lr * (1.f + cosf(3.14159265f * (float)step / (float)std::max<long long>(1, steps_total)));
       s->adam_t++;
@@ -1006,12 +1019,9 @@ extern "C" int sur_train(sur_t *s, const float *X, const float *Y, int n, int ep
       k_adam<<<egrid(s->nparam), 256, 0, s->stream>>>(s->w, s->g, s->m, s->v, s->w16, s->nparam, lr_t, b1, b2, eps, c1,
                                                        c2);
       e = cudaGetLastError();
+      const int done = b0 / batch + 1;
+      if (e == cudaSuccess && (done - read == keep || done == per_epoch)) read_losses(done);
     }
-    // the copy also keeps the host's order from being reshuffled before it is uploaded
-    if (e == cudaSuccess) e = cudaMemcpyAsync(lp.data(), dL, lp.size() * 4, cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    double lsum = 0;
-    for (int q = 0; q < per_epoch; q++) lsum += loss_of(s, lp.data() + (size_t)q * LOSS_PARTS, std::min(batch, n - q * batch));
     if (epoch_loss) epoch_loss[ep] = (float)(lsum / per_epoch);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);

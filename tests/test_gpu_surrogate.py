@@ -215,3 +215,23 @@ def test_weight_gradients_at_ragged_shapes(n, l0, chans):
         k = int(np.prod(sh))
         assert cosine(g[o:o + k], gq[o:o + k]) >= 0.99, name
         o += k
+
+
+def test_epoch_loss_over_many_minibatches():
+    """An epoch of more minibatches than the device keeps loss partials for: the
+    mean of the cases' losses.  At a learning rate of 1e-20 weights of 1e-8 and more
+    stay (the biases, zero at first, are set to 0.01), so loss_grad gives each case's loss by the same kernels (mean in double over the
+    FP32 losses: 1e-6)."""
+    from paper_2302_13907_gb300.binding import Surrogate
+    rng = np.random.default_rng(2)
+    n = 2049
+    X = rng.standard_normal((n, 4)).astype(np.float32)
+    Y = rng.standard_normal((n, 8, 64)).astype(np.float32)
+    with Surrogate(max_batch=8, in_dim=4, h1=32, h2=32, l0=16, chans=(16, 16, 8), out_ch=8) as s:
+        w = s.params()
+        w[np.abs(w) < 1e-8] = 0.01
+        s.set_params(w)
+        hist = s.train(X, Y, epochs=2, batch=1, lr=1e-20, seed=3)
+        assert np.array_equal(w, s.params())
+        ref = np.mean([s.loss_grad(X[q:q + 1], Y[q:q + 1])[0] for q in range(n)])
+    assert np.abs(hist - ref).max() <= 1e-6 * ref, (hist, ref)

@@ -47,3 +47,19 @@ out["calls"] = calls
             assert done, log
             assert any(x[0] == "wait" and x[1] == main and x[2] == done[0][1] for x in log[done[0][0]:]), log
     assert left > 20  # failures with work on a side stream
+
+
+def test_training_memory_does_not_grow_with_the_number_of_minibatches():
+    """Beside the data and the order of the cases, an epoch takes a few MB however
+    many minibatches it has."""
+    r = run(NET + """
+n = 40000
+X, Y = np.zeros((n, 4), np.float32), np.zeros((n, 8, 64), np.float32)
+with net() as s:
+    before = fake.fake_used()
+    fake.fake_peak(1)
+    s.train(X, Y, epochs=0, batch=1)
+    out["extra"] = fake.fake_peak(0) - before - X.nbytes - Y.nbytes - 4 * n
+    out["left"] = fake.fake_used() - before
+""")
+    assert r["extra"] <= 8 << 20 and r["left"] == 0, r
