@@ -59,7 +59,8 @@ struct simr_s {
   SideStream rec_side{};
   bool rec_pending = false;
   int big_zone = 0;
-  bool zone_streams = false, forced = false;  // forced: opts.tile names the split codes
+  // zone_streams: the zones of a half on parallel streams; one_launch: in one launch
+  bool zone_streams = false, one_launch = false;
   int vel_code = 0, str_code = 0;  // split codes of every zone's halves
   sim_grid_t grid{};
   int NR = 0, NZ = 0, NZp = 0, M = 0;
@@ -140,12 +141,14 @@ double dirichlet(int N, double t) {
 
 bool pow2_in(int n) { return n == 4 || n == 8 || n == 16 || n == 32 || n == 64; }
 
-// split codes of a grid whose largest zone fills the GPU (the 20 m well; the
+// split codes of a grid whose largest zone fills the GPU (the 20 m well; several
 // zones then run on parallel streams): interior and radial layer marched along
 // theta, 1375 us a step of the 20 m well where the best tile-by-tile pair (2285 and
 // 2334) takes 1449.  A smaller grid (a 1.6 m crop, several handles side by side) runs
 // all zones of a half in one launch of the batched kernel: 126 us a step of the
-// 136 x 32 x 1330 crop, 176 with two launches per zone and half.
+// 136 x 32 x 1330 crop, 176 with two launches per zone and half; with a largest zone
+// of 7.7 M cells 295 and 335.  A single zone is no exception: 13.5 M cells take 317 us
+// in one launch, 285 in two a half, 51.8 M cells 1149 and 983.
 constexpr int REFINED_VEL_CODE = 2324, REFINED_STR_CODE = 2324;
 constexpr long long ZONE_STREAM_CELLS = 8LL << 20;
 // opts.tile of a refined handle: 0, or a split code or pair code whose halves
@@ -163,7 +166,7 @@ bool refined_tile_ok(int t) {
 // such handles usually run side by side already and the extra streams there
 // cost more than they overlap.
 cudaError_t zones_half(simr_t *h, int code, int parts) {
-  if (!h->zone_streams && !h->forced) return launch_batch_split(0, parts == 1, h->kps.data(), (int)h->kps.size(), h->stream);
+  if (h->one_launch) return launch_batch_split(0, parts == 1, h->kps.data(), (int)h->kps.size(), h->stream);
   const int nz = h->zone_streams ? (int)h->kps.size() : 1;
   if (!h->zone_streams) {  // one after another on the handle's stream
     cudaError_t e = cudaSuccess;
@@ -540,6 +543,7 @@ extern "C" int simr_create(const sim_grid_t *grid, const simr_zones_t *zones, co
       if (cells > most) most = cells, h->big_zone = m;
     }
     h->zone_streams = M > 1 && most >= ZONE_STREAM_CELLS;
+    h->one_launch = !opts->tile && most < ZONE_STREAM_CELLS;
     for (int k = 0; k < M - 1; k++) {
       if ((e = cudaStreamCreateWithFlags(&h->zs[k], cudaStreamNonBlocking)) != cudaSuccess ||
           (e = cudaEventCreateWithFlags(&h->zjoin[k], cudaEventDisableTiming)) != cudaSuccess)
@@ -556,7 +560,6 @@ extern "C" int simr_create(const sim_grid_t *grid, const simr_zones_t *zones, co
   // zero state of zone 0 with the source off (the state stays zero)
   h->vel_code = opts->tile ? split_vel_code(opts->tile) : REFINED_VEL_CODE;
   h->str_code = opts->tile ? split_str_code(opts->tile) : REFINED_STR_CODE;
-  h->forced = opts->tile != 0;
   if (opts->tile) {
     KParams dry = h->kps[0];
     dry.src_i = -1;
