@@ -523,11 +523,14 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
       pick = rt;
     }
   }
-  if (!forced && pick_v >= 0 && best_v + best_s < best) {  // the split family's best halves win
-    pick = pick_v == pick_s ? pick_v : pick_v * 10000 + pick_s;
-    // the halves within 3 % of the best ones, paired and timed again as they
-    // run: whole steps in a captured graph, the edge launches on the side
-    // stream (the times above are of separate launches, three at a time)
+  if (!forced && pick_v >= 0) {
+    // The times above are of separate launches, three at a time, in which every
+    // launch costs some microseconds that a captured chunk does not pay.  So the
+    // families are compared as they run, by whole steps in a captured graph, the
+    // edge launches on the side stream: the halves within 3 % of the best ones,
+    // paired; the best of the other kernels where it was ahead of the halves (44 x
+    // 8 x 256 cells, FP16-SR: the sweep kernel, one launch, was, and takes 23.1 us a
+    // step against 14.3); the one-pass step.
     auto near = [](std::vector<std::pair<float, int>> t, float b) {
       std::sort(t.begin(), t.end());
       std::vector<int> out;
@@ -536,30 +539,41 @@ static int autotune(sim_t *h, int kernel, int forced, int *best_rt) {
       return out;
     };
     const std::vector<int> nv = near(times_v, best_v), ns = near(times_s, best_s);
+    const int other = best <= best_v + best_s ? pick : -1;
     KParams dry = h->kp;
     dry.src_i = -1;
     float best_step = INFINITY;
     cudaError_t e = cudaSuccess;
-    if (pass_ok || nv.size() * ns.size() > 1)
+    auto step_time = [&](int code, auto step) {
+      float ms = 0;
+      if (e == cudaSuccess) e = time_graph(h, a, b, &ms, step);
+      if (e == cudaSuccess && ms < best_step) best_step = ms, pick = code;
+    };
+    pick = pick_v == pick_s ? pick_v : pick_v * 10000 + pick_s;
+    if (pass_ok || other >= 0 || nv.size() * ns.size() > 1)
       for (int v : nv)
         for (int c : ns) {
           const int code = v == c ? v : v * 10000 + c;
-          float ms = 0;
-          if (e == cudaSuccess)
-            e = time_graph(h, a, b, &ms, [&](int) { return launch_split_family(h->stencil_storage, code, dry, h->stream, nullptr); });
-          if (e == cudaSuccess && ms < best_step) best_step = ms, pick = code;
+          step_time(code, [&](int) { return launch_split_family(h->stencil_storage, code, dry, h->stream, nullptr); });
         }
     h->split_rt = pick;
-    // the one-pass step against the best pair: ahead from some 3 M cells on (88 x 22
-    // x 1527 cells 75 us a step against 79), behind where a march is short and the
-    // state stays in L2 anyway (70 x 16 x 320 cells 18.8 us against 14.6)
+    if (other >= 0) {
+      const int rc = is_march(other) ? build_march_maps(h, other) : is_sweep(other) ? SIM_OK : build_maps(h, other);
+      if (rc) return rc;
+      FusedParams fp[2] = {h->fp[0], h->fp[1]};
+      fp[0].k.src_i = fp[1].k.src_i = -1;
+      step_time(other, [&](int r) {
+        return is_march(other)   ? launch_march(h->storage, other, h->mmaps, dry, h->status, h->stream, nullptr)
+               : is_sweep(other) ? launch_sweep(h->stencil_storage, other, dry, h->vdone, h->status, 0, -1, h->stream)
+                                 : launch_fused_any(h->storage, other, h->maps[r & 1], fp[r & 1], h->stream);
+      });
+    }
+    // the one-pass step is ahead from some 3 M cells on (88 x 22 x 1527 cells 75 us a
+    // step against 79), behind where a march is short and the state stays in L2
+    // anyway (70 x 16 x 320 cells 18.8 us against 14.6)
     if (pass_ok)
-      for (int code : {4001, 4101, 4201, 4301}) {
-        float ms = 0;
-        if (2 * pass_runs(code) > h->grid.nth || e != cudaSuccess) continue;
-        e = time_graph(h, a, b, &ms, [&](int r) { return launch_pass_step(h, code, r & 1, true, nullptr); });
-        if (e == cudaSuccess && ms < best_step) best_step = ms, pick = code;
-      }
+      for (int code : {4001, 4101, 4201, 4301})
+        step_time(code, [&](int r) { return launch_pass_step(h, code, r & 1, true, nullptr); });
     if (e != cudaSuccess) {
       cudaEventDestroy(a);
       cudaEventDestroy(b);

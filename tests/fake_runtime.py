@@ -19,6 +19,7 @@ import ctypes, json, sys
 sys.path.insert(0, {root!r})
 fake = ctypes.CDLL({lib!r}, ctypes.RTLD_GLOBAL)
 fake.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]
+fake.fake_launch_cost.argtypes = [ctypes.c_double]
 fake.fake_total.argtypes = [ctypes.c_size_t]
 fake.fake_fail_launch.argtypes = [ctypes.c_long]
 fake.fake_used.restype = fake.fake_peak.restype = ctypes.c_size_t

@@ -112,3 +112,23 @@ with B.Simulation(sc, max_steps=65536, mem_cap=out["bytes"] + set_bytes - 256) a
 """)
     assert r["capped"] == [1, r["bytes"]] and r["short"] == [1, r["bytes"]]
     assert r["free"] == 6 and r["room"] == 6
+
+
+@pytest.mark.parametrize("kernel,kind,us,storage", [
+    ("sweep", 5, 30.0, "f32"), ("sweep", 5, 90.0, "f16sr"), ("fused", 2, 30.0, "f16")])
+def test_families_are_compared_as_they_run(kernel, kind, us, storage):
+    """A kernel of fewer launches that leads where each launch costs something by
+    itself is picked only if it also leads in a captured graph."""
+    r = run(WELLS + f"""
+def pick(sc):
+    with B.Simulation(sc, storage={storage!r}) as s:
+        s.step(4)
+        return s.config()[0]
+fake.fake_launch_cost(40.0)  # split halves: one launch of 10 us each, with stochastic rounding three
+fake.fake_cost(b"pass_step", 1000.0)
+fake.fake_cost({kernel!r}.encode(), {us})
+out["slower in a graph"] = pick(well())
+fake.fake_cost({kernel!r}.encode(), 2.0)
+out["faster in a graph"] = pick(well(nz=84))
+""")
+    assert r == {"slower in a graph": 1, "faster in a graph": kind}
