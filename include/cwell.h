@@ -402,8 +402,8 @@ const char *simb_last_error(const simb_t *b);
  * rows per zone, the radial PML inside the last zone (row0 <= nr - 2); FP32
  * storage; any source kind, placed on the nodes of the zone that holds it
  * (the transverse force off the axis and the torsion ring not on a zone's
- * first row, SIM_EUNSUPPORTED).  Every zone runs the split kernels, code
- * 2324 (largest zone of at least 8 Mi cells; the
+ * first row, SIM_EUNSUPPORTED).  Every zone runs the split kernels: code 2275
+ * with a largest zone of at least 8 Mi cells, 2324 from 38 Mi on (the
  * zones of a half then run on parallel streams); on smaller grids all zones of
  * a half share one launch.  opts.tile may name a 22xx / 23xx split code or pair
  * code instead (SIM_EINVAL otherwise; small grids then run zone after zone).

@@ -141,15 +141,20 @@ double dirichlet(int N, double t) {
 
 bool pow2_in(int n) { return n == 4 || n == 8 || n == 16 || n == 32 || n == 64; }
 
-// split codes of a grid whose largest zone fills the GPU (the 20 m well; several
-// zones then run on parallel streams): interior and radial layer marched along
-// theta, 1375 us a step of the 20 m well where the best tile-by-tile pair (2285 and
-// 2334) takes 1449.  A smaller grid (a 1.6 m crop, several handles side by side) runs
-// all zones of a half in one launch of the batched kernel: 126 us a step of the
-// 136 x 32 x 1330 crop, 176 with two launches per zone and half; with a largest zone
-// of 7.7 M cells 295 and 335.  A single zone is no exception: 13.5 M cells take 317 us
-// in one launch, 285 in two a half, 51.8 M cells 1149 and 983.
-constexpr int REFINED_VEL_CODE = 2324, REFINED_STR_CODE = 2324;
+// A grid whose largest zone fills the GPU runs every zone's halves with a split
+// code, several zones on parallel streams.  The interior is marched along theta.
+// The radial layer's march pays only where its runs fill the GPU several times over
+// (us a step by the largest zone's cells, 2324 with it against 2275 without: 8.4 M
+// 279 / 270, 8.7 M 282 / 266, 15.8 M 456 / 442, 25.8 M 693 / 696, 28.4 M 776 / 776,
+// 32.8 M 889 / 880, 36.6 M 1007 / 997, 41.0 M 1099 / 1111, 51.6 M 1359 / 1379; the
+// best tile-by-tile pair, 2285 and 2334: 281 at 8.4 M, 1451 at 51.6 M).
+// A smaller grid (a 1.6 m crop, several handles side by side) runs all zones of a
+// half in one launch of the batched kernel: 126 us a step of the 136 x 32 x 1330
+// crop, 176 with two launches per zone and half; with a largest zone of 7.7 M cells
+// 295 and 335.  A single zone is no exception: 13.5 M cells take 317 us in one
+// launch, 282 in two a half, 51.8 M cells 1149 and 983.
+constexpr int REFINED_CODE = 2275, REFINED_CODE_LARGE = 2324;
+constexpr long long LARGE_ZONE_CELLS = 38LL << 20;
 constexpr long long ZONE_STREAM_CELLS = 8LL << 20;
 // opts.tile of a refined handle: 0, or a split code or pair code whose halves
 // are interior / edge (22xx) or three-way (23xx) split codes
@@ -536,8 +541,8 @@ extern "C" int simr_create(const sim_grid_t *grid, const simr_zones_t *zones, co
     h->kps.push_back(p);
   }
   // the zones' streams: the largest zone stays on the handle's stream
+  long long most = -1;
   {
-    long long most = -1;
     for (int m = 0; m < M; m++) {
       const long long cells = (long long)h->kps[m].nth * (h->kps[m].i_hi - h->kps[m].i_lo) * NZ;
       if (cells > most) most = cells, h->big_zone = m;
@@ -558,8 +563,9 @@ extern "C" int simr_create(const sim_grid_t *grid, const simr_zones_t *zones, co
   }
   // the zones' split codes; a forced one is tried once per half on the still
   // zero state of zone 0 with the source off (the state stays zero)
-  h->vel_code = opts->tile ? split_vel_code(opts->tile) : REFINED_VEL_CODE;
-  h->str_code = opts->tile ? split_str_code(opts->tile) : REFINED_STR_CODE;
+  const int code = opts->tile ? opts->tile : most >= LARGE_ZONE_CELLS ? REFINED_CODE_LARGE : REFINED_CODE;
+  h->vel_code = split_vel_code(code);
+  h->str_code = split_str_code(code);
   if (opts->tile) {
     KParams dry = h->kps[0];
     dry.src_i = -1;

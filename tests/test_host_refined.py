@@ -31,3 +31,13 @@ def test_a_zone_that_fills_the_gpu_has_its_own_launches(rows):
     rows_of = 28 + (rows[0] if rows else 0)
     assert not kernels(rows_of, 64, nz, rows)[0]
     assert kernels(rows_of, 64, nz - 16, rows)[0]
+
+
+@pytest.mark.parametrize("rows", [[], [8]])
+def test_the_radial_layer_is_marched_in_large_zones(rows):
+    """The interior of every zone with launches of its own is marched along theta,
+    the radial layer from 38 Mi cells on."""
+    skip = rows[0] if rows else 0
+    assert kernels(28 + skip, 64, 4096 + 4, rows) == (False, True, False)
+    assert kernels(147 + skip, 64, 4096 + 4, rows) == (False, True, False)   # x 151 rows
+    assert kernels(148 + skip, 64, 4096 + 4, rows) == (False, True, True)    # x 152 rows
