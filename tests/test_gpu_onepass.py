@@ -138,3 +138,29 @@ def test_refused_where_it_cannot_run():
         with pytest.raises(SimError) as ei:
             sim(sc, **kw)
         assert ei.value.code == SIM_EINVAL
+
+
+def test_largest_material_table():
+    """2196 materials fill the shared memory beside the staged planes; one more is
+    refused for a tile asked for and runs the other kernels under AUTO."""
+    from paper_2302_13907_gb300.binding import SIM_EINVAL, SimError
+    for n_mat in (2196, 2197):
+        sc = scenario(11, 8, 14, 141, steps=40)
+        m = sc.medium
+        rng = np.random.default_rng(n_mat)
+        q = np.arange(n_mat) % 4
+        f = 1 + 1e-4 * (np.arange(n_mat) // 4)
+        m.rho, m.vp, m.vs = m.rho[q], m.vp[q] * f, m.vs[q] * f
+        m.cell_id = rng.integers(0, n_mat, size=m.grid.shape).astype(np.uint16)
+        m.cell_id[:, 0] = 0
+        if n_mat == 2197:
+            with pytest.raises(SimError) as ei:
+                sim(sc, tile=4001)
+            assert ei.value.code == SIM_EINVAL
+        o = oracle.Oracle(sc)
+        with sim(sc, tile=4001 if n_mat == 2196 else 0) as s:
+            assert (s.config()[0] == 6) == (n_mat == 2196)
+            start(sc, s, o)
+            s.step(sc.steps)
+            o.step(sc.steps)
+            fields_match(s, o)

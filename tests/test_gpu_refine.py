@@ -128,3 +128,12 @@ def test_refined_longitudinal_force_and_torsion_ring(kind, r0):
                       z=np.array([0.05, 0.1, 0.12]))
     sc = W.Scenario("refined-sources", med, W.Source(r=r0, theta=0.7, z=0.08, f0=60e3, kind=kind), rec, steps=160)
     _compare(sc, [4, 8], steps=160)
+
+
+@pytest.mark.parametrize("tile", [2324, 2275])
+@pytest.mark.parametrize("rows,nth", [([4, 8], 16), ([3, 6, 10], 32)])
+def test_refined_zones_marched_along_theta(tile, rows, nth):
+    """The codes large zones run: the march on zones with ghost rows at either
+    side, both halves, against the oracle as above."""
+    sc = _ragged(seed=6, nth=nth, kind=0, src_r=0.0305)
+    _compare(sc, rows, steps=120, tile=tile)

@@ -104,3 +104,34 @@ def test_slab_rejects_misaligned_bounds():
     with pytest.raises(SimError) as ei:
         Simulation(sc, slab=(0, 101))
     assert ei.value.code == SIM_EINVAL
+
+
+@pytest.mark.parametrize("tile", [2324, 2275])
+@pytest.mark.parametrize("ws", [2, 3])
+def test_marched_slabs(tile, ws):
+    """Slabs whose halves are marched along theta: as close to the oracle as the
+    undivided well on the same code (bars as above)."""
+    import torch
+    from paper_2302_13907_gb300.binding import Simulation
+    sc = _scenario()
+    p = slabs.plan(sc.grid.NZ, ws)
+    stream = torch.cuda.current_stream().cuda_stream
+    o = oracle.Oracle(sc)
+    o.step(sc.steps)
+    with Simulation(sc, kernel="split", tile=tile, stream=stream) as whole:
+        whole.step(sc.steps)
+        ref = {f: whole.field(f) for f in oracle.FIELDS}
+    engines = [slabs.SimSlab(sc, p, r, stream=stream, tile=tile) for r in range(ws)]
+    try:
+        slabs.run_local(engines, p, sc.steps)
+        torch.cuda.synchronize()
+        for r, e in enumerate(engines):
+            s0, s1 = p.owned(r)
+            for f in oracle.FIELDS:
+                scale = np.abs(o.field(f)).max()
+                b = o.field(f)[:, :, s0:s1]
+                d = np.abs(e.sim.field(f)[:, :, s0 - e.sim.l0:s1 - e.sim.l0] - b).max()
+                assert d <= 4 * np.abs(ref[f][:, :, s0:s1] - b).max() + 2e-5 * scale, (r, f, d / scale)
+    finally:
+        for e in engines:
+            e.sim.close()
