@@ -373,7 +373,9 @@ int simb_sync(simb_t *b);
 int simb_traces(simb_t *b, int which, float *out, size_t cap, int *n_rec, int *n_steps);
 int simb_read_field(simb_t *b, int which, int field, float *out, size_t n);
 
-/* Number of cases, work items (tiles) and blocks of one shared launch. */
+/* Number of cases, tiles of the shared cases in a half step (one block each) and
+ * blocks of the largest of its launches (up to 64 cases share one; 1 without
+ * shared cases). */
 int simb_config(const simb_t *b, int *n_cases, long long *work_items, int *grid_blocks);
 /* Cases on their own launches and the parallel streams they run on. */
 int simb_layout(const simb_t *b, int *own_cases, int *branches);

@@ -437,7 +437,7 @@ class BatchSimulation:
         return out
 
     def config(self):
-        """(cases, work items per launch, persistent blocks per launch)."""
+        """(cases, tiles of the shared cases in a half step, blocks of its largest launch)."""
         n, w, g = ctypes.c_int(), ctypes.c_longlong(), ctypes.c_int()
         self._chk(self.L.simb_config(self.h, ctypes.byref(n), ctypes.byref(w), ctypes.byref(g)))
         return n.value, w.value, g.value

@@ -20,7 +20,7 @@ struct simb_s {
   std::vector<KParams> kp;        // the cases' kernel parameters (host: they travel as kernel parameters)
   std::vector<int> shared, own;   // cases in the shared launches / on their own tuned launches
   RParams *d_rp = nullptr;
-  long long total = 0;  // blocks of the shared cases in one half step
+  long long total = 0, widest = 0;  // blocks of the shared cases in one half step; of its largest launch
   int graph_chunk = 64, steps_done = 0;
   // parallel streams for the own-launch cases: case own[q] runs on branch[q % nbranch]
   static constexpr int MAX_BRANCH = 4;
@@ -201,6 +201,7 @@ extern "C" int simb_create(int n, const sim_grid_t *grids, const sim_medium_t *m
   o.graph_chunk = -1;
   o.timing = 0;
   size_t used = 0;
+  long long launch = 0;  // blocks of the launch being filled with up to BATCH_MAX cases
   for (int c = 0; c < n; c++) {
     if (opts->mem_cap) o.mem_cap = opts->mem_cap > used ? opts->mem_cap - used : 1;
     const long long cells =
@@ -218,6 +219,8 @@ extern "C" int simb_create(int n, const sim_grid_t *grids, const sim_medium_t *m
     if (blocks > 0x7fffffffLL)
       return bail(bfail(b, SIM_EINVAL, "case " + std::to_string(c) + ": more work items than a 32-bit index holds"));
     b->total += blocks;
+    launch = (b->shared.size() - 1) % BATCH_MAX == 0 ? blocks : launch + blocks;
+    b->widest = std::max(b->widest, launch);
   }
   b->kp.resize(n);
   std::vector<RParams> rp(n);
@@ -318,7 +321,7 @@ extern "C" int simb_config(const simb_t *b, int *n_cases, long long *work_items,
   if (!b) return SIM_EINVAL;
   if (n_cases) *n_cases = (int)b->cases.size();
   if (work_items) *work_items = b->total;
-  if (grid_blocks) *grid_blocks = (int)std::min<long long>(std::max<long long>(1, b->total), 0x7fffffff);
+  if (grid_blocks) *grid_blocks = (int)std::min<long long>(std::max<long long>(1, b->widest), 0x7fffffff);
   return SIM_OK;
 }
 

@@ -2,7 +2,7 @@
 // its host logic without a GPU.  Loaded into the global symbol scope before the
 // library (fake_runtime.py).  Device memory is host memory; kernels do not run.
 // A launch moves the clock on by its kernel's cost and is written to a log with
-// its stream, as are event records and waits.  Refused as by the real runtime:
+// its stream and grid, as are event records and waits.  Refused as by the real runtime:
 // more dynamic shared memory than the kernel was granted, and more device memory
 // than there is.  A test can let a coming launch fail.
 #include <cuda.h>
@@ -106,7 +106,7 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **, s
     }
   if (capture) capture->cost += us;
   else now += us + launch_us;
-  log("launch", s, nullptr, name.c_str());
+  log("launch", s, (void *)(size_t)grid.x, name.c_str());
   return cudaSuccess;
 }
 cudaError_t cudaFuncSetAttribute(const void *f, enum cudaFuncAttribute a, int v) {
