@@ -351,6 +351,18 @@ __device__ __forceinline__ float stretch_reg(float &psi, float a, float b, float
 // spread it.
 __device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 
+// The z derivative of a cell that has radial memory variables.  In the general body
+// a select between it and its stretched value keeps the compiler from fusing its
+// product into the sum that follows; in a body without z memory variables the
+// product is rounded by itself in BF16 and FP16 storage, so that both give the same
+// bits.  (FP32, where no rounding to storage amplifies a last bit, and the
+// stochastic rounding, whose layer has always run this body, keep it fused.)
+template <typename T, bool LAYER>
+__device__ __forceinline__ float z_diff(float dz, float idz) {
+  if constexpr (LAYER && (std::is_same<T, __nv_bfloat16>::value || std::is_same<T, __half>::value)) return __fmul_rn(dz, idz);
+  else return dz * idz;
+}
+
 // cell k of a row of the interior whose aligned pair of cells lies clear of the z
 // PML: the cells that a kernel with two cells per thread gives to the lean body
 __device__ __forceinline__ bool lean_pair(const KParams &p, int i, int k) {
@@ -516,7 +528,7 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
     if (im) {
       const float dr = srr_e - m_srr[e], dz = srz_e - srz_m1;
       const float q = 0.5f * (srr_e + m_srr[e]) - 0.5f * (spp_e + m_spp[e]) + (srp_e - jm_srp[e]) * idth;
-      float Dr = dr * idr, Q = q * inv_ri, Dz = dz * idz;
+      float Dr = dr * idr, Q = q * inv_ri, Dz = z_diff<T, ZIN && !LEAN>(dz, idz);
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vr[e], abr.x, abr.y, Dr) : stretch(p.psr[R_VR] + cr + e, abr.x, abr.y, Dr));
         Q = (PRE ? stretch_reg(uq_vr[e], abq.x, abq.y, Q) : stretch(p.psr[Q_VR] + cr + e, abq.x, abq.y, Q));
@@ -529,7 +541,7 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
     {
       const float s1 = p_srp[e];
       const float dr = s1 - srp_e, q = (s1 + srp_e) + (jp_spp[e] - spp_e) * idth, dz = spz_e - spz_m1;
-      float Dr = dr * idr, Q = q * inv_rh, Dz = dz * idz;
+      float Dr = dr * idr, Q = q * inv_rh, Dz = z_diff<T, ZIN && !LEAN>(dz, idz);
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vp[e], abr.z, abr.w, Dr) : stretch(p.psr[R_VP] + cr + e, abr.z, abr.w, Dr));
         Q = (PRE ? stretch_reg(uq_vp[e], abq.z, abq.w, Q) : stretch(p.psr[Q_VP] + cr + e, abq.z, abq.w, Q));
@@ -544,7 +556,7 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
       const float dr = s1 - srz_e, dz = (e < NV - 1 ? a_szz[e + 1] : szz_k4) - szz_e;
       const float q = lean ? mul_add2(0.5f, s1 + srz_e, spz_e - jm_spz[e], idth)
                            : 0.5f * (s1 + srz_e) + (spz_e - jm_spz[e]) * idth;
-      float Dr = dr * idr, Q = q * inv_rh, Dz = dz * idz;
+      float Dr = dr * idr, Q = q * inv_rh, Dz = z_diff<T, ZIN && !LEAN>(dz, idz);
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vz[e], abr.z, abr.w, Dr) : stretch(p.psr[R_VZ] + cr + e, abr.z, abr.w, Dr));
         Q = (PRE ? stretch_reg(uq_vz[e], abq.z, abq.w, Q) : stretch(p.psr[Q_VZ] + cr + e, abq.z, abq.w, Q));
@@ -735,7 +747,7 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
       const float vr1 = p_vr[e];
       float err = (vr1 - vr_e) * idr;
       float epp = ((vp_e - jm_vp[e]) * idth + 0.5f * (vr_e + vr1)) * inv_rh;
-      float ezz = (vz_e - vz_m1) * idz;
+      float ezz = z_diff<T, ZIN && !LEAN>(vz_e - vz_m1, idz);
       if (rp) {
         err = (PRE ? stretch_reg(ur_rr[e], abr.z, abr.w, err) : stretch(p.psr[R_ERR] + cr + e, abr.z, abr.w, err));
         epp = (PRE ? stretch_reg(uq_pp[e], abq.z, abq.w, epp) : stretch(p.psr[Q_EPP] + cr + e, abq.z, abq.w, epp));
@@ -770,7 +782,7 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
       // s_rz at (r_i, theta_j, z_{k+1/2})
       if (ZIN || k + 1 < NZ) {
         const float dz = vr_e1 - vr_e, dr = vz_e - m_vz[e];
-        float gz = dz * idz, gr = dr * idr;
+        float gz = z_diff<T, ZIN && !LEAN>(dz, idz), gr = dr * idr;
         if (zp) gz = (PRE ? stretch_reg(uz_rz[e], abz.z, abz.w, gz) : stretch(p.psz[Z_GRZ] + czrow + kz, abz.z, abz.w, gz));
         if (rp) gr = (PRE ? stretch_reg(ur_rz[e], abr.x, abr.y, gr) : stretch(p.psr[R_GRZ] + cr + e, abr.x, abr.y, gr));
         const float mu = mu_harm(imu_m[e] + imu_c[e] + imu_m[e + 1] + imu_c[e + 1]);
@@ -781,7 +793,7 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
     if (ZIN || k + 1 < NZ) {
       const float dz = vp_e1 - vp_e;
       float Q = (jp_vz[e] - vz_e) * idth * inv_rh;
-      float gz = dz * idz;
+      float gz = z_diff<T, ZIN && !LEAN>(dz, idz);
       if (rp) Q = (PRE ? stretch_reg(uq_pz[e], abq.z, abq.w, Q) : stretch(p.psr[Q_GPZ] + cr + e, abq.z, abq.w, Q));
       if (zp) gz = (PRE ? stretch_reg(uz_pz[e], abz.z, abz.w, gz) : stretch(p.psz[Z_GPZ] + czrow + kz, abz.z, abz.w, gz));
       const float mu = mu_harm(imu_c[e] + imu_j[e] + imu_c[e + 1] + imu_j[e + 1]);

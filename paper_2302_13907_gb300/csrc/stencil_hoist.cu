@@ -95,13 +95,23 @@ Regions region_tiles(const KParams &p, int r0, int za, int zb) {
   return q;
 }
 
-template <int NV, int NVE>
+// first row of the radial layer's tiles.  Stochastic rounding decides by the last
+// bits of FP32, so its layer keeps the cells each body has always had: the radial
+// body whole tiles of rows and of 128 z cells (radial_cells_step), of which the first
+// may start above the layer.
+template <typename T>
+int layer_row(const KParams &p) {
+  const int r = std::min(p.nr, p.NR);
+  return std::is_same<T, half_sr>::value ? r / HB_Y * HB_Y : r;
+}
+
+template <typename T, int NV, int NVE>
 Regions regions(const KParams &p) {
   int za = (p.pml_z + 3) / 4 * 4, zb = std::max(za, (p.NZ - p.pml_z - 1) / 4 * 4);
   constexpr int W = NV * HB_X;
   if (za % W > W - W / 4) za = (za + W - 1) / W * W;
   if (zb % W < W / 4) zb = zb / W * W;
-  return region_tiles<NV, NVE>(p, std::min(p.nr, p.NR), za, std::max(za, zb));
+  return region_tiles<NV, NVE>(p, layer_row<T>(p), za, std::max(za, zb));
 }
 
 // cell group of this thread in interior tile t (theta fastest, then r, then z); false: nothing to do
@@ -138,8 +148,18 @@ __device__ __forceinline__ void lean_cells_step(const KParams &p, int j, int i, 
   if (VEL) vel_hoist_body<T, NV, true>(p, j, i, k0);
   else str_hoist_body<T, NV, true>(p, j, i, k0);
 }
+// the 128 z cells around k0 lie clear of both layers and the z end
+__device__ __forceinline__ bool whole_tile(const KParams &p, int k0) {
+  const int t = k0 / 128 * 128;
+  return t >= p.pml_z && t + 128 <= p.NZ - p.pml_z - 1;
+}
 template <typename T, int NV, bool VEL>
 __device__ __forceinline__ void radial_cells_step(const KParams &p, int j, int i, int k0, const OutSet *out = nullptr) {
+  if constexpr (std::is_same<T, half_sr>::value)
+    if (!whole_tile(p, k0)) {
+      hoist_cells<T, NV, VEL, true>(p, j, i, k0);
+      return;
+    }
   if (VEL) vel_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
   else str_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
 }
@@ -347,7 +367,7 @@ cudaError_t launch_batch_t(const KParams *cases, int n_cases, cudaStream_t s) {
       bp.inner[c] = (int)inner;
       if (c == n) break;
       bp.cases[c] = cases[c0 + c];
-      bp.q[c] = regions<BATCH_NV, BATCH_NVE>(cases[c0 + c]);
+      bp.q[c] = regions<T, BATCH_NV, BATCH_NVE>(cases[c0 + c]);
       edge += bp.q[c].ends + bp.q[c].radial;
       inner += bp.q[c].interior;
       if (edge + inner > 0x7fffffffLL || bp.q[c].ends * (HB_X * HB_Y) > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -454,7 +474,7 @@ inline bool fits(const Regions &q) { return q.interior + q.radial + q.ends * (HB
 
 template <typename T, int NV, int MINB_IN, int MODE, int NVE, int MINB_R, int MINB_E, int PFE = 0>
 cudaError_t launch_split_t(const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts) {
-  const Regions q = regions<NV, NVE>(p);
+  const Regions q = regions<T, NV, NVE>(p);
   if (!fits(q)) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
   if (parts & 1) {
@@ -472,7 +492,7 @@ cudaError_t launch_split_t(const KParams &p, cudaStream_t s, cudaEvent_t *ev, in
 
 template <typename T, int NV, int NVE, int MINB>
 cudaError_t launch_one_t(const KParams &p, cudaStream_t s, cudaEvent_t *ev, int parts) {
-  const Regions q = regions<NV, NVE>(p);
+  const Regions q = regions<T, NV, NVE>(p);
   if (!fits(q)) return cudaErrorInvalidValue;
   const int grid = (int)(q.ends + q.radial + q.interior);
   if (parts & 1) {
@@ -586,7 +606,7 @@ cudaError_t launch_hoist_st(int code, const KParams &p, cudaStream_t s, cudaEven
 void set_side_stream(const SideStream *ss) { g_side = ss; }
 
 long long batch_blocks(const KParams &p) {
-  const Regions q = regions<BATCH_NV, BATCH_NVE>(p);
+  const Regions q = regions<float, BATCH_NV, BATCH_NVE>(p);
   return q.ends + q.radial + q.interior;
 }
 

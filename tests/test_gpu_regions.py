@@ -124,3 +124,60 @@ def test_no_trace_of_the_cut_in_the_fields(tile, storage, steps, nz, pml_z):
             x, y = a.field(n), b.field(n)
             assert np.abs(y).max() > 0, n
             assert np.array_equal(x, y), (n, np.flatnonzero((x != y).any((0, 1))))
+
+
+def _noisy_well(nr, pml_r, nz, pml_z, steps):
+    g = W.Grid(nr=nr, nth=6, nz=nz, pml_r=pml_r, pml_z=pml_z, dr=0.004, dz=0.003)
+    rng = np.random.default_rng(nz)
+    mats = [W.FLUID, W.STEEL, W.CEMENT, W.ROCK]
+    cid = rng.integers(0, len(mats), size=g.shape).astype(np.uint16)
+    cid[:, 0, :] = 0
+    med = W.Medium(g, cid, *(np.array([m[q] for m in mats]) for q in range(3)))
+    sc = W.Scenario("cut", med, W.Source(r=0.009, theta=2.0, z=0.012, f0=60e3), W.on_axis_receivers([0.0]), steps=steps)
+    v = {n: rng.standard_normal(g.shape).astype(np.float32) / (1000 * 1500) for n in ("vr", "vp", "vz")}
+    v["vr"][:, 0] = 0
+    v["vz"][:, :, -1] = 0
+    return sc, v
+
+
+@pytest.mark.parametrize("tile", [2204, 2216, 2224, 2256, 2275, 2285, 2304, 2314, 2324])
+@pytest.mark.parametrize("storage", ["bf16", "f16"])
+@pytest.mark.parametrize("nr,pml_r,nz,pml_z", [(9, 5, 146, 3), (10, 3, 300, 9), (8, 4, 252, 4)])
+def test_radial_layer_in_16_bit_storage(tile, storage, nr, pml_r, nz, pml_z):
+    """The radial layer's own bodies, wherever their region starts and ends, give the
+    bits of the general body (2106), every field."""
+    from paper_2302_13907_gb300.binding import Simulation
+    sc, v = _noisy_well(nr, pml_r, nz, pml_z, 160)
+    with Simulation(sc, kernel="split", tile=tile, storage=storage) as a, \
+            Simulation(sc, kernel="split", tile=2106, storage=storage) as b:
+        for n in v:
+            a.set_field(n, v[n])
+            b.set_field(n, v[n])
+        a.step(sc.steps)
+        b.step(sc.steps)
+        for n in oracle.FIELDS:
+            x, y = a.field(n), b.field(n)
+            assert np.abs(y).max() > 0, n
+            assert np.array_equal(x, y), (n, np.flatnonzero((x != y).any((0, 2))))
+
+
+@pytest.mark.parametrize("tile", [2304, 2305, 2314, 2324, 2335])
+@pytest.mark.parametrize("nr,pml_r,nz,pml_z,crc", [
+    (10, 5, 300, 9, 0x25d6cab3),    # two rows above the layer share its first tile
+    (9, 3, 500, 15, 0xe9d95514),
+    (11, 4, 250, 3, 0xa9d32746),
+])
+def test_stochastic_rounding_keeps_its_bits(tile, nr, pml_r, nz, pml_z, crc):
+    """FP16 with stochastic rounding, 60 steps: the fields of the kernels that cut
+    their regions at whole tiles of 4 rows x 128 z cells (all 23xx codes gave these)."""
+    import zlib
+    from paper_2302_13907_gb300.binding import Simulation
+    sc, v = _noisy_well(nr, pml_r, nz, pml_z, 60)
+    with Simulation(sc, kernel="split", tile=tile, storage="f16sr") as s:
+        for n in v:
+            s.set_field(n, v[n])
+        s.step(60)
+        got = 0
+        for n in oracle.FIELDS:
+            got = zlib.crc32(np.ascontiguousarray(s.field(n)).tobytes(), got)
+    assert got == crc
