@@ -134,7 +134,11 @@ typedef struct {
   int pml_off;        /* 1: rigid walls with no PML (energy-conserving closure) */
   int graph_chunk;    /* steps per captured CUDA graph; 0 = 64; < 0 = no graph */
   void *cuda_stream;  /* cudaStream_t to enqueue on; NULL = a stream owned by the handle */
-  size_t mem_cap;     /* bytes of device memory the handle may take; 0 = no cap */
+  size_t mem_cap;     /* bytes of device memory the handle may take; 0 = no cap.  SIM_KERNEL_AUTO
+                         takes a second set of fields and, for the volumetric source, of memory
+                         variables; point forces and torsion (FP32) take the fields alone, if they
+                         are at most a third of the free memory and fit under the cap, and give
+                         them back unless the one-pass step is picked */
   int max_steps;      /* trace capacity in steps; 0 = 65536 */
   int kernel;         /* SIM_KERNEL_* */
   int timing;         /* 1: bracket each kernel launch with CUDA events (no graph) */
@@ -268,8 +272,8 @@ double sim_dt(const sim_t *h);
 int sim_steps_done(const sim_t *h);
 size_t sim_device_bytes(const sim_t *h);
 
-/* Path the handle runs: *kernel = SIM_KERNEL_SPLIT, SIM_KERNEL_FUSED or
- * SIM_KERNEL_MARCH; *tile_rows = the tile code chosen by the autotuner (or
+/* Path the handle runs: *kernel = SIM_KERNEL_SPLIT, SIM_KERNEL_FUSED,
+ * SIM_KERNEL_MARCH, SIM_KERNEL_SWEEP or SIM_KERNEL_ONEPASS; *tile_rows = the tile code chosen by the autotuner (or
  * forced by opts.tile): r (< 100) for the fused kernel with r rows per block,
  * 100 + r for its four-cells-per-thread variant; 1000 + 100 r + J for the
  * marching kernels with r rows per block and runs of J theta planes; 2000 for
@@ -299,13 +303,15 @@ size_t sim_device_bytes(const sim_t *h);
  * cells 2.5 and 2 chunks behind; m = 1, 3 add an L2 prefetch of each block's
  * next velocity item).
  * 4000 + 100 m + d the one-pass step (kernel = AUTO, FP32, a second field set
- * in memory, at least 4 rows and 32 z cells away from the PML, up to about 3500
- * materials; SIM_EINVAL otherwise): both halves of the lean cells in one kernel,
+ * in memory, at least 4 rows and 32 z cells away from the PML, up to 2196
+ * materials, which fill a block's 227 KB of shared memory beside the staged planes;
+ * SIM_EINVAL otherwise): both halves of the lean cells in one kernel,
  * theta in d runs (1 .. nth, at most 32) per tile, m = 0, 2: one block per SM
  * walks the tiles, 1, 3: one block per tile; the other cells with split bodies of
  * two (m = 0, 1) or four (2, 3; the radial layer marched along theta) cells per
  * thread.
- * opts.tile accepts every code listed here. */
+ * opts.tile accepts every code listed here; the tuner tries the one-pass step with
+ * d = 1. */
 int sim_config(const sim_t *h, int *kernel, int *tile_rows);
 
 /* Test hook of the failure path of the sweep kernel (SIM_KERNEL_SWEEP), the
@@ -324,8 +330,9 @@ int sim_config(const sim_t *h, int *kernel, int *tile_rows);
 int sim_set_wait_test(sim_t *h, long long wait_cycles, int withhold_chunk);
 
 /* Kernel timings gathered with opts.timing = 1: for kernel slot q
- * (0 = fused or sweep kernel, or the velocity kernel of the split and marching paths,
- * 1 = their stress kernel, 2 = receivers), total milliseconds and launch count so far.
+ * (0 = fused or sweep kernel, the one-pass kernel with the launches beside it, or the
+ * velocity kernel of the split and marching paths, 1 = their stress kernel or the
+ * stresses after the one-pass kernel, 2 = receivers), total milliseconds and launch count so far.
  * Synchronises. */
 int sim_kernel_time(sim_t *h, int q, double *ms, long *launches);
 

@@ -431,7 +431,7 @@ void launch_interior(const KParams &p, const Regions &q, cudaStream_t s) {
   dim3 blk(HB_X, HB_Y);
   if constexpr (MODE == 2) {
     static_assert(NV == 4, "four cells per thread");
-    constexpr int MB = sizeof(T) == 2 && !VEL ? MINB - 1 : MINB;  // without spills: 3 stress blocks, 4 velocity blocks
+    constexpr int MB = sizeof(T) == 2 && !VEL ? MINB - 1 : MINB;  // 16 bits: 3 stress, 4 velocity blocks (at most 8 bytes spilled)
     if (can_run<T>(p)) launch_run<T, MB, VEL, false, false>(p, q, OutSet{}, s);
     else hoist_interior<T, NV, 4, VEL><<<(int)q.interior, blk, 0, s>>>(p, q);
   } else if constexpr (MODE == 1) hoist_interior_pf<T, NV, MINB, VEL><<<wave(q.interior, MINB), blk, 0, s>>>(p, q);

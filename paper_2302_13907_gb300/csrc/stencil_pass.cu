@@ -29,7 +29,8 @@
 // + 100 m + d), the tiles left over in more and shorter ones; one block per SM
 // walks the (tile, run) items, its ring running on from item to item (m even),
 // or every item has its own block (m odd: no fixed share of the items per SM,
-// but a pipeline fill per item).  The tuner picks.
+// but a pipeline fill per item).  The tuner times both with theta in one run (d = 1);
+// other d are for opts.tile.
 //
 // Measured: 196 x 64 x 8224 cells 1.27 ms a launch (74 bytes a cell: 5.5 TB/s)
 // where the split halves take 0.83 + 1.03 ms on the same cells; the step with its

@@ -456,7 +456,6 @@ __global__ void k_adam(float *w, const float *g, float *m, float *v, __nv_bfloat
   }
 }
 
-// gather rows of the device training set into a minibatch
 // per case b: num[b] = sum (y - y0)^2 and den[b] = sum y0^2 over its `per`
 // outputs (one block per case, fixed-order tree in the block)
 __global__ void __launch_bounds__(256) k_diff_norms(const float *y, const float *y0, long long per, float *num,
@@ -485,6 +484,7 @@ __global__ void __launch_bounds__(256) k_diff_norms(const float *y, const float 
   }
 }
 
+// gather rows of the device training set into a minibatch
 __global__ void k_gather(const float *src, const int *idx, int n, long long row, float *dst) {
   GRID_STRIDE(q, (long long)n * row) dst[q] = src[(long long)idx[q / row] * row + q % row];
 }
