@@ -225,7 +225,7 @@ __device__ __forceinline__ void stown(T *p, const float (&v)[NV]) {
 // on the same grid.  One path for every value, nothing on the conversion unit
 // but the packing: with floor, int-to-float and a branch for zeros a FP16-SR step of
 // the 196 x 64 x 1056 crop took 453 us tile by tile, with this 387 (marched along theta
-// and with the reciprocal unit 294: hoist_run.cuh).
+// and with the reciprocal unit 288: hoist_run.cuh).
 struct SrKey {
   unsigned long long zc, zs;  // (common part + 1) G, S G
   int k0;
@@ -352,16 +352,28 @@ __device__ __forceinline__ float stretch_reg(float &psi, float a, float b, float
 // spread it.
 __device__ __forceinline__ float mul_add2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 
-// The z derivative of a cell that has radial memory variables.  In the general body
-// a select between it and its stretched value keeps the compiler from fusing its
-// product into the sum that follows; in a body without z memory variables the
-// product is rounded by itself in BF16 and FP16 storage, so that both give the same
-// bits.  (FP32, where no rounding to storage amplifies a last bit, and the
-// stochastic rounding, whose layer has always run this body, keep it fused.)
+// The z derivative D of a cell of the radial layer, and its sum with the other terms.
+// In the general body a select between D and its stretched value keeps the compiler
+// from fusing D's product into the sum that follows; the body without z memory
+// variables (LAYER) rounds the product by itself in 16-bit storage, so that both give
+// the same bits.  In FP32, where no rounding to storage amplifies a last bit, it stays
+// fused.  Stochastic rounding shows every last bit, so its cells keep what they have
+// always had: in whole tiles of the layer (whole_tile, layer_row) the product is
+// fused, in the others not.
 template <typename T, bool LAYER>
 __device__ __forceinline__ float z_diff(float dz, float idz) {
-  if constexpr (LAYER && (std::is_same<T, __nv_bfloat16>::value || std::is_same<T, __half>::value)) return __fmul_rn(dz, idz);
+  if constexpr (LAYER && sizeof(T) == 2) return __fmul_rn(dz, idz);
   else return dz * idz;
+}
+template <typename T, bool LAYER>
+__device__ __forceinline__ float z_sum(float a, float D, float dz, float idz, bool whole) {
+  if constexpr (LAYER && std::is_same<T, half_sr>::value) return whole ? __fmaf_rn(dz, idz, a) : a + D;
+  else return a + D;
+}
+// the 128 z cells around k0 lie clear of both layers and the z end
+__device__ __forceinline__ bool whole_tile(const KParams &p, int k0) {
+  const int t = k0 / 128 * 128;
+  return t >= p.pml_z && t + 128 <= p.NZ - p.pml_z - 1;
 }
 
 // cell k of a row of the interior whose aligned pair of cells lies clear of the z
@@ -405,6 +417,9 @@ __device__ __forceinline__ void zero_ids(int (&o)[NV]) {
 template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN, bool PAIRS = false>
 __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, const int i, const int k0,
                                                const OutSet *out = nullptr) {
+  // a body of the radial layer; with stochastic rounding also of rows that share its first tile
+  constexpr bool LAYER = ZIN && !LEAN, SR_LAYER = LAYER && std::is_same<T, half_sr>::value;
+  const bool whole = SR_LAYER && whole_tile(p, k0);
   void *const *fo = out ? out->f : p.f;
   const int nth = p.nth, NR = p.NR, NZ = p.NZ;
   const long long NZp = p.NZp, pl = p.plane;
@@ -521,7 +536,7 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
     const bool zp = zl && (k < pz || k >= NZ - pz);
     const int kz = k < pz ? k : k - (NZ - 2 * pz);
     const float4 abz = zp ? __ldg(p.ab_z + k) : z4();
-    const bool lean = PAIRS && lean_pair(p, i, k);
+    const bool lean = SR_LAYER ? !whole && i < p.nr : PAIRS && lean_pair(p, i, k);
     const float srr_e = a_srr[e], spp_e = a_spp[e], srp_e = a_srp[e];
     const float srz_e = a_srz[e], spz_e = a_spz[e], szz_e = a_szz[e];
     const float srz_m1 = e ? a_srz[e - 1] : srz_km, spz_m1 = e ? a_spz[e - 1] : spz_km;
@@ -529,26 +544,26 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
     if (im) {
       const float dr = srr_e - m_srr[e], dz = srz_e - srz_m1;
       const float q = 0.5f * (srr_e + m_srr[e]) - 0.5f * (spp_e + m_spp[e]) + (srp_e - jm_srp[e]) * idth;
-      float Dr = dr * idr, Q = q * inv_ri, Dz = z_diff<T, ZIN && !LEAN>(dz, idz);
+      float Dr = dr * idr, Q = q * inv_ri, Dz = z_diff<T, LAYER>(dz, idz);
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vr[e], abr.x, abr.y, Dr) : stretch(p.psr[R_VR] + cr + e, abr.x, abr.y, Dr));
         Q = (PRE ? stretch_reg(uq_vr[e], abq.x, abq.y, Q) : stretch(p.psr[Q_VR] + cr + e, abq.x, abq.y, Q));
       }
       if (zp) Dz = (PRE ? stretch_reg(uz_vr[e], abz.x, abz.y, Dz) : stretch(p.psz[Z_VR] + czrow + kz, abz.x, abz.y, Dz));
-      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_ri)) : Dr + Q + Dz;
+      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_ri)) : z_sum<T, LAYER>(Dr + Q, Dz, dz, idz, whole);
       out_r[e] += vel_coef(dtv, rho_m[e] + rho_c[e]) * t;
     }
     // v_phi at (r_{i+1/2}, theta_{j+1/2}, z_k)
     {
       const float s1 = p_srp[e];
       const float dr = s1 - srp_e, q = (s1 + srp_e) + (jp_spp[e] - spp_e) * idth, dz = spz_e - spz_m1;
-      float Dr = dr * idr, Q = q * inv_rh, Dz = z_diff<T, ZIN && !LEAN>(dz, idz);
+      float Dr = dr * idr, Q = q * inv_rh, Dz = z_diff<T, LAYER>(dz, idz);
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vp[e], abr.z, abr.w, Dr) : stretch(p.psr[R_VP] + cr + e, abr.z, abr.w, Dr));
         Q = (PRE ? stretch_reg(uq_vp[e], abq.z, abq.w, Q) : stretch(p.psr[Q_VP] + cr + e, abq.z, abq.w, Q));
       }
       if (zp) Dz = (PRE ? stretch_reg(uz_vp[e], abz.x, abz.y, Dz) : stretch(p.psz[Z_VP] + czrow + kz, abz.x, abz.y, Dz));
-      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_rh)) : Dr + Q + Dz;
+      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_rh)) : z_sum<T, LAYER>(Dr + Q, Dz, dz, idz, whole);
       out_p[e] += vel_coef(dtv, rho_c[e] + rho_j[e]) * t;
     }
     // v_z at (r_{i+1/2}, theta_j, z_{k+1/2}), k + 1 < NZ
@@ -557,13 +572,13 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
       const float dr = s1 - srz_e, dz = (e < NV - 1 ? a_szz[e + 1] : szz_k4) - szz_e;
       const float q = lean ? mul_add2(0.5f, s1 + srz_e, spz_e - jm_spz[e], idth)
                            : 0.5f * (s1 + srz_e) + (spz_e - jm_spz[e]) * idth;
-      float Dr = dr * idr, Q = q * inv_rh, Dz = z_diff<T, ZIN && !LEAN>(dz, idz);
+      float Dr = dr * idr, Q = q * inv_rh, Dz = z_diff<T, LAYER>(dz, idz);
       if (rp) {
         Dr = (PRE ? stretch_reg(ur_vz[e], abr.z, abr.w, Dr) : stretch(p.psr[R_VZ] + cr + e, abr.z, abr.w, Dr));
         Q = (PRE ? stretch_reg(uq_vz[e], abq.z, abq.w, Q) : stretch(p.psr[Q_VZ] + cr + e, abq.z, abq.w, Q));
       }
       if (zp) Dz = (PRE ? stretch_reg(uz_vz[e], abz.z, abz.w, Dz) : stretch(p.psz[Z_VZ] + czrow + kz, abz.z, abz.w, Dz));
-      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_rh)) : Dr + Q + Dz;
+      const float t = lean ? __fmaf_rn(dz, idz, mul_add2(dr, idr, q, inv_rh)) : z_sum<T, LAYER>(Dr + Q, Dz, dz, idz, whole);
       out_z[e] += vel_coef(dtv, rho_c[e] + rho_c[e + 1]) * t;
     }
   }
@@ -601,6 +616,9 @@ __device__ __forceinline__ void vel_hoist_body(const KParams &p, const int j, co
 template <typename T, int NV, bool LEAN, bool PRE = false, bool ZIN = LEAN, bool CG = false, bool PAIRS = false>
 __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, const int i, const int k0,
                                                const OutSet *out = nullptr) {
+  // a body of the radial layer; with stochastic rounding also of rows that share its first tile
+  constexpr bool LAYER = ZIN && !LEAN, SR_LAYER = LAYER && std::is_same<T, half_sr>::value;
+  const bool whole = SR_LAYER && whole_tile(p, k0);
   void *const *fo = out ? out->f : p.f;
   const int nth = p.nth, NR = p.NR, NZ = p.NZ;
   const long long NZp = p.NZp, pl = p.plane;
@@ -739,7 +757,7 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
     const bool zp = zl && (k < pz || k >= NZ - pz);
     const int kz = k < pz ? k : k - (NZ - 2 * pz);
     const float4 abz = zp ? __ldg(p.ab_z + k) : z4();
-    const bool lean = PAIRS && lean_pair(p, i, k);
+    const bool lean = SR_LAYER ? !whole && i < p.nr : PAIRS && lean_pair(p, i, k);
     const float vr_e = a_vr[e], vp_e = a_vp[e], vz_e = a_vz[e];
     const float vr_e1 = e < NV - 1 ? a_vr[e + 1] : vr_k4, vp_e1 = e < NV - 1 ? a_vp[e + 1] : vp_k4;
     const float vz_m1 = e ? a_vz[e - 1] : vz_km;
@@ -748,7 +766,7 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
       const float vr1 = p_vr[e];
       float err = (vr1 - vr_e) * idr;
       float epp = ((vp_e - jm_vp[e]) * idth + 0.5f * (vr_e + vr1)) * inv_rh;
-      float ezz = z_diff<T, ZIN && !LEAN>(vz_e - vz_m1, idz);
+      float ezz = z_diff<T, LAYER>(vz_e - vz_m1, idz);
       if (rp) {
         err = (PRE ? stretch_reg(ur_rr[e], abr.z, abr.w, err) : stretch(p.psr[R_ERR] + cr + e, abr.z, abr.w, err));
         epp = (PRE ? stretch_reg(uq_pp[e], abq.z, abq.w, epp) : stretch(p.psr[Q_EPP] + cr + e, abq.z, abq.w, epp));
@@ -783,22 +801,23 @@ __device__ __forceinline__ void str_hoist_body(const KParams &p, const int j, co
       // s_rz at (r_i, theta_j, z_{k+1/2})
       if (ZIN || k + 1 < NZ) {
         const float dz = vr_e1 - vr_e, dr = vz_e - m_vz[e];
-        float gz = z_diff<T, ZIN && !LEAN>(dz, idz), gr = dr * idr;
+        float gz = z_diff<T, LAYER>(dz, idz), gr = dr * idr;
         if (zp) gz = (PRE ? stretch_reg(uz_rz[e], abz.z, abz.w, gz) : stretch(p.psz[Z_GRZ] + czrow + kz, abz.z, abz.w, gz));
         if (rp) gr = (PRE ? stretch_reg(ur_rz[e], abr.x, abr.y, gr) : stretch(p.psr[R_GRZ] + cr + e, abr.x, abr.y, gr));
         const float mu = mu_harm(imu_m[e] + imu_c[e] + imu_m[e + 1] + imu_c[e + 1]);
-        orz[e] += dts * mu * (lean ? mul_add2(dz, idz, dr, idr) : gz + gr);
+        orz[e] += dts * mu * (lean ? mul_add2(dz, idz, dr, idr) : SR_LAYER ? z_sum<T, LAYER>(gr, gz, dz, idz, whole) : gz + gr);
       }
     }
     // s_phiz at (r_{i+1/2}, theta_{j+1/2}, z_{k+1/2})
     if (ZIN || k + 1 < NZ) {
       const float dz = vp_e1 - vp_e;
       float Q = (jp_vz[e] - vz_e) * idth * inv_rh;
-      float gz = z_diff<T, ZIN && !LEAN>(dz, idz);
+      float gz = z_diff<T, LAYER>(dz, idz);
       if (rp) Q = (PRE ? stretch_reg(uq_pz[e], abq.z, abq.w, Q) : stretch(p.psr[Q_GPZ] + cr + e, abq.z, abq.w, Q));
       if (zp) gz = (PRE ? stretch_reg(uz_pz[e], abz.z, abz.w, gz) : stretch(p.psz[Z_GPZ] + czrow + kz, abz.z, abz.w, gz));
       const float mu = mu_harm(imu_c[e] + imu_j[e] + imu_c[e + 1] + imu_j[e + 1]);
-      opz[e] += dts * mu * (lean ? __fmaf_rn(dz, idz, __fmul_rn(__fmul_rn(jp_vz[e] - vz_e, idth), inv_rh)) : Q + gz);
+      opz[e] += dts * mu * (lean ? __fmaf_rn(dz, idz, __fmul_rn(__fmul_rn(jp_vz[e] - vz_e, idth), inv_rh)) 
+                                 : z_sum<T, LAYER>(Q, gz, dz, idz, whole));
     }
   }
   const SrKey sk = body_key<T>(p, j, i, k0);

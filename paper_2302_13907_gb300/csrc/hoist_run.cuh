@@ -9,7 +9,7 @@
 // the theta neighbours once (they are the present values of the plane before or
 // after), and with 32-bit offsets and the material table in shared memory takes
 // 420.  196 x 64 x 1056 cells, BF16: 217 us a step tile by tile, 193 here;
-// FP16-SR 342 and 285 (294 since its radial layer takes whole tiles again); FP32 on 136 x
+// FP16-SR 342 and 285 (288 with its layer in whole tiles, z_sum); FP32 on 136 x
 // 32 x 3104 cells 294 and 269.  Its interior
 // launches reach 66 and 57 % of the DRAM throughput (53 and 46 % tile by tile); what
 // is left is issue slots (57 to 61 % busy) and the start of every run.

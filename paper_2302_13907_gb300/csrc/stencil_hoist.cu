@@ -96,9 +96,9 @@ Regions region_tiles(const KParams &p, int r0, int za, int zb) {
 }
 
 // first row of the radial layer's tiles.  Stochastic rounding decides by the last
-// bits of FP32, so its layer keeps the cells each body has always had: the radial
-// body whole tiles of rows and of 128 z cells (radial_cells_step), of which the first
-// may start above the layer.
+// bits of FP32, so its layer keeps the order of sums that each cell has always had,
+// by whole tiles of rows and of 128 z cells (z_sum); the first tile of rows may start
+// above the layer.
 template <typename T>
 int layer_row(const KParams &p) {
   const int r = std::min(p.nr, p.NR);
@@ -148,18 +148,8 @@ __device__ __forceinline__ void lean_cells_step(const KParams &p, int j, int i, 
   if (VEL) vel_hoist_body<T, NV, true>(p, j, i, k0);
   else str_hoist_body<T, NV, true>(p, j, i, k0);
 }
-// the 128 z cells around k0 lie clear of both layers and the z end
-__device__ __forceinline__ bool whole_tile(const KParams &p, int k0) {
-  const int t = k0 / 128 * 128;
-  return t >= p.pml_z && t + 128 <= p.NZ - p.pml_z - 1;
-}
 template <typename T, int NV, bool VEL>
 __device__ __forceinline__ void radial_cells_step(const KParams &p, int j, int i, int k0, const OutSet *out = nullptr) {
-  if constexpr (std::is_same<T, half_sr>::value)
-    if (!whole_tile(p, k0)) {
-      hoist_cells<T, NV, VEL, true>(p, j, i, k0);
-      return;
-    }
   if (VEL) vel_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
   else str_hoist_body<T, NV, false, true, true>(p, j, i, k0, out);
 }
