@@ -882,7 +882,6 @@ extern "C" int sur_forward(sur_t *s, const float *X, int n, float *Y) {
   SCK(s, cudaSetDevice(s->device));
   const sur_cfg_t &c = s->cfg;
   const int Lf = L_out(s);
-  std::vector<float> tmp((size_t)s->max_batch * Lf * c.out_ch);
   for (int b0 = 0; b0 < n; b0 += s->max_batch) {
     const int nb = std::min(s->max_batch, n - b0);
     SCK(s, cudaMemcpyAsync(s->xb, X + (size_t)b0 * c.in_dim, (size_t)nb * c.in_dim * 4, cudaMemcpyHostToDevice,
